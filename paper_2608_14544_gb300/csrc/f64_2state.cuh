@@ -4,6 +4,8 @@
 // whole step of one walker (Verlet, phase, transition test) and the walker's
 // observable contributions.
 #pragma once
+#include <type_traits>
+
 #include "kernels.h"
 
 namespace qcl {
@@ -34,29 +36,6 @@ struct Ad2 {
   double a, b, r, c2, s2;
 };
 
-template <int NP>
-__device__ __forceinline__ Ad2 decomp(const DevModel* M, const double* R, int n) {
-  double a = M->a0, b = M->b0;
-#pragma unroll
-  for (int j = 0; j < NP; ++j)
-    if (j < n) {
-      a += M->a[j] * R[j];
-      b += M->b[j] * R[j];
-    }
-  Ad2 d;
-  d.a = a;
-  d.b = b;
-  d.r = sqrt(a * a + b * b);
-  if (d.r > 0.0) {
-    d.c2 = a / d.r;
-    d.s2 = b / d.r;
-  } else {
-    d.c2 = 1.0;
-    d.s2 = 0.0;
-  }
-  return d;
-}
-
 __device__ __forceinline__ void half_angle(const Ad2& d, double& c, double& s) {
   if (d.r == 0.0) {
     c = 1.0;
@@ -72,24 +51,7 @@ __device__ __forceinline__ void half_angle(const Ad2& d, double& c, double& s) {
   }
 }
 
-__device__ __forceinline__ double sigma(int idx) { return idx ? 1.0 : -1.0; }
-
-// P += dt/2 F_ab(R), F_j = -k_j R_j - s_j - 1/2 (sig_a + sig_b)(a_j cos2t + b_j sin2t)
-template <int NP>
-__device__ __forceinline__ void half_kick(const DevModel* M, const double* R, double* P, int n,
-                                          const Ad2& d, int al, int be, double dt) {
-  const double sab = 0.5 * (sigma(al) + sigma(be));
-#pragma unroll
-  for (int j = 0; j < NP; ++j)
-    if (j < n) {
-      const double F =
-          -M->k[j] * R[j] - (M->s[j] + sab * (M->a[j] * d.c2 + M->b[j] * d.s2));
-      P[j] += 0.5 * dt * F;
-    }
-}
-
-// Global-memory variant for large mode counts: the same arithmetic reading
-// R, P from the SoA arrays (stride nt).
+// The decomposition at R read from the SoA arrays (stride nt).
 __device__ __forceinline__ Ad2 decomp_g(const DevModel* M, const double* R, int64_t nt, int n) {
   double a = M->a0, b = M->b0;
   for (int j = 0; j < n; ++j) {
@@ -195,144 +157,299 @@ __device__ __forceinline__ void sample_walker_f64(const DevModel* __restrict__ M
   ab = (uint16_t)(al | (be << 8));
 }
 
-// Outcome of one step's transition test: event 0 (none), 1 (first index) or
-// 2 (second index); the weight factor num / den that the event carries
-// (m <- m * num / den: A_e / p_hat_e for an event, 1 / (1 - sum p_hat) for
-// none), the event's quarter turns, and whether a degenerate gap was met.
-struct Step64 {
-  int ev;
-  double num, den;
-  int dq;
+// --------------------------------------------------------------- FP64 step --
+// The FP64 unit is the narrow resource here (2 lanes per clock per SM; the
+// kernels below keep it 80-90 % busy), so a step is written for few FP64
+// operations: per-mode constants made on the host and read as constant-bank
+// operands, one reciprocal square root in place of a square root and two
+// divisions, the decomposition at R_n carried from the step before, the
+// spin-boson form without the terms that are zero there, thresholds and weight
+// factors from integers, signs and selections in integer registers.  Every
+// operation is an explicit round-to-nearest one, so that the bits do not
+// depend on where the step is inlined (one launch or several, moving or
+// spawning walkers).
+
+// Per-mode and per-launch constants (kernel parameter; NC modes).
+template <int NC>
+struct Coef64 {
+  double hk[NC], hs[NC];  // dt/2 k_j, dt/2 s_j
+  double dtm[NC];         // dt / M_j
+  double a[NC], b[NC];    // d a / d R_j, d b / d R_j
+  double am[NC], bm[NC];  // a_j / M_j, b_j / M_j
+  double a0, b0;
+  double hdt;    // dt / 2
+  double wph;    // dt / hbar: dt/2 (w_n + w_{n+1}) = +-wph (r_n + r_{n+1}) off the diagonal
+  double cg;     // event amplitude |A_e| = |dt g|: cg Av ir^2 (spin-boson form,
+                 // cg = -b0 dt/2), cg (a Bv - b Av) ir^2 (cg = dt/2), or cg b (diabatic,
+                 // cg = dt / hbar)
+  double kamp;   // hop_scale 2^24
+  uint32_t tmax2;  // floor(floor(p_max 2^24) / 2)
+  int32_t n;
+};
+
+template <int NC>
+inline void make_coef64(const DevModel& h, double dt, Coef64<NC>& c) {
+  for (int j = 0; j < NC; ++j) {
+    const bool on = j < h.n;
+    c.hk[j] = on ? 0.5 * dt * h.k[j] : 0.0;
+    c.hs[j] = on ? 0.5 * dt * h.s[j] : 0.0;
+    c.dtm[j] = on ? dt / h.mass[j] : 0.0;
+    c.a[j] = on ? h.a[j] : 0.0;
+    c.b[j] = on ? h.b[j] : 0.0;
+    c.am[j] = on ? h.a[j] / h.mass[j] : 0.0;
+    c.bm[j] = on ? h.b[j] / h.mass[j] : 0.0;
+  }
+  c.a0 = h.a0;
+  c.b0 = h.b0;
+  c.hdt = 0.5 * dt;
+  c.wph = dt / h.hbar;
+  c.cg = h.repr == QCL_REPR_DIABATIC ? dt / h.hbar : (h.kind == 0 ? -0.5 * h.b0 * dt : 0.5 * dt);
+  c.kamp = h.hop_scale * kP24;
+  c.tmax2 = (uint32_t)std::floor(h.p_max * kP24) >> 1;
+  c.n = h.n;
+}
+
+// A positive normal float as a double, from its bits (no FP64 or conversion
+// instruction).
+__device__ __forceinline__ double widen_normal(float x) {
+  const uint32_t u = __float_as_uint(x);
+  return __hiloint2double((int)((u >> 3) + ((1023u - 127u) << 20)), (int)(u << 29));
+}
+
+// 1 / i for an integer 0 < i <= 2^24: the FP32 reciprocal and two Newton steps
+// r <- r + r (1 - i r) (relative error 2^-23 -> 2^-46 -> the last rounding).
+__device__ __forceinline__ double rcp_int(double i, uint32_t iu) {
+  float f;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint2float_rn(iu)));
+  double r = widen_normal(f);
+  r = __fma_rn(r, __fma_rn(-i, r, 1.0), r);
+  return __fma_rn(r, __fma_rn(-i, r, 1.0), r);
+}
+
+// An integer below 2^32 as a double (bits of 2^52 + i, less 2^52).
+__device__ __forceinline__ double int_double(uint32_t i) {
+  return __dadd_rn(__hiloint2double(0x43300000, (int)i), -0x1p52);
+}
+
+// 1 / sqrt(x) for x in the normal range: the hardware approximation y (relative
+// error e/2, e = 1 - x y^2) and one third-order step y (1 + e/2 + 3/8 e^2).
+__device__ __forceinline__ double rsqrt64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+  return __fma_rn(__fma_rn(e, 0.375, 0.5), __dmul_rn(e, y), y);
+}
+
+// The decomposition a walker carries between steps: a(R), b(R), r, 1/r^2 (0
+// where the gap is degenerate, which sets the coupling to 0), cos and sin
+// 2theta, and whether the gap is degenerate.
+struct Dec64 {
+  double a, b, r, ir2, c2, s2;
   bool deg;
 };
 
+// (r^2 below (kDegTol / 2)^2: the exact square root and quotients, theta = 0
+// at r = 0.)
+template <int KIND, bool DIA>
+__device__ __forceinline__ void decompose64(Dec64& d) {
+  d.deg = false;
+  if (DIA) return;
+  const double r2 = __fma_rn(d.a, d.a, __dmul_rn(d.b, d.b));
+  const double ir = rsqrt64(r2);
+  d.r = __dmul_rn(r2, ir);
+  d.ir2 = __dmul_rn(ir, ir);
+  d.c2 = __dmul_rn(d.a, ir);
+  if (KIND == 1) d.s2 = __dmul_rn(d.b, ir);
+  if (__double_as_longlong(r2) < __double_as_longlong(0.25 * kDegTol * kDegTol)) {
+    d.deg = true;
+    d.r = sqrt(r2);
+    d.ir2 = 0.0;
+    d.c2 = d.r > 0.0 ? d.a / d.r : 1.0;
+    if (KIND == 1) d.s2 = d.r > 0.0 ? d.b / d.r : 0.0;
+  }
+}
+
+// Outcome of one step's transition test: event 0 (none), 1 (first index) or
+// 2 (second index); the factor the event puts on the weight (A_e / p_hat_e for
+// an event, 1 / (1 - sum p_hat) for none); the event's quarter turns.
+struct Step64 {
+  int ev;
+  double factor;
+  int dq;
+};
+
+// P += dt/2 F_ab for one mode with hu = dt/2 sab cos 2theta, hv = dt/2 sab sin
+// 2theta (diabatic: hu = -dt/2 sab).
+template <int KIND, bool DIA>
+__device__ __forceinline__ double kick64(double hk, double hs, double a, double b, double R,
+                                         double P, double hu, double hv) {
+  P = __fma_rn(-hk, R, P);
+  if (KIND == 1) P = __dadd_rn(P, -hs);
+  P = __fma_rn(-hu, a, P);
+  if (KIND == 1 && !DIA) P = __fma_rn(-hv, b, P);
+  return P;
+}
+
 // One step n -> n+1 of one two-state walker in FP64: velocity Verlet on the
 // pair's mean force (adiabatic: Hellmann-Feynman diagonal; diabatic: the
-// diagonal of W), the trapezoid phase, and the transition test with the
-// walker's hop stream `stream` (Philox word n & 3 of block n >> 2).  R and P
-// are read and written at Rg[j * stride], Pg[j * stride].
-template <int NP, bool DIA>
-__device__ __forceinline__ Step64 walker_step_f64(const DevModel* __restrict__ M, double* Rg,
-                                                  double* Pg, int64_t stride, int n, int al,
-                                                  int be, double& phi, double dt, uint64_t seed,
-                                                  uint64_t stream, int64_t step) {
-  Ad2 d0, d1;
+// diagonal of W), the trapezoid phase, and the transition test with the hop
+// word `y` (24 bits).  R and P of NP > 0 modes in registers, or (NP = 0) at
+// Rg[j * stride], Pg[j * stride] in two passes; d is the decomposition at R_n
+// on entry and at R_{n+1} on return; deg reports a degenerate gap at either.
+template <int NP, int NC, int KIND, bool DIA>
+__device__ __forceinline__ Step64 walker_step_f64(const Coef64<NC>& c, double* R, double* P,
+                                                  int64_t stride, Dec64& d, int al, int be,
+                                                  double& phi, uint32_t y, bool& deg) {
+  // dt/2 (sig_a + sig_b)/2 and dt/hbar (sig_a - sig_b)/2 of the pair
+  const bool same = al == be;
+  const double hsab = same ? (al ? c.hdt : -c.hdt) : 0.0;
+  const double wab = same ? 0.0 : (al ? c.wph : -c.wph);
+  const double hu = DIA ? -hsab : __dmul_rn(hsab, d.c2);
+  const double hv = (KIND == 1 && !DIA) ? __dmul_rn(hsab, d.s2) : 0.0;
+  const double w0 = DIA ? d.a : d.r;
+  deg = d.deg;
+  d.a = c.a0;
+  d.b = c.b0;
   double Av = 0.0, Bv = 0.0;
   if constexpr (NP > 0) {
-    double R[NP], P[NP];
 #pragma unroll
     for (int j = 0; j < NP; ++j)
-      if (j < n) {
-        R[j] = Rg[(int64_t)j * stride];
-        P[j] = Pg[(int64_t)j * stride];
+      if (NP <= 4 || j < c.n) {
+        P[j] = kick64<KIND, DIA>(c.hk[j], c.hs[j], c.a[j], c.b[j], R[j], P[j], hu, hv);
+        R[j] = __fma_rn(c.dtm[j], P[j], R[j]);
+        d.a = __fma_rn(c.a[j], R[j], d.a);
+        if (KIND == 1) d.b = __fma_rn(c.b[j], R[j], d.b);
       }
-    d0 = decomp<NP>(M, R, n);
-    if (DIA) {  // the diagonal force is the kick's with cos 2theta = -1, sin 2theta = 0
-      d0.c2 = -1.0;
-      d0.s2 = 0.0;
-    }
-    half_kick<NP>(M, R, P, n, d0, al, be, dt);
+    decompose64<KIND, DIA>(d);
+    const double hu2 = DIA ? hu : __dmul_rn(hsab, d.c2);
+    const double hv2 = (KIND == 1 && !DIA) ? __dmul_rn(hsab, d.s2) : 0.0;
 #pragma unroll
     for (int j = 0; j < NP; ++j)
-      if (j < n) R[j] += dt * P[j] / M->mass[j];
-    d1 = decomp<NP>(M, R, n);
-    if (DIA) {
-      d1.c2 = -1.0;
-      d1.s2 = 0.0;
-    }
-    half_kick<NP>(M, R, P, n, d1, al, be, dt);
-#pragma unroll
-    for (int j = 0; j < NP; ++j)
-      if (j < n) {
+      if (NP <= 4 || j < c.n) {
+        P[j] = kick64<KIND, DIA>(c.hk[j], c.hs[j], c.a[j], c.b[j], R[j], P[j], hu2, hv2);
         if (!DIA) {
-          Av += M->a[j] * (P[j] / M->mass[j]);
-          Bv += M->b[j] * (P[j] / M->mass[j]);
+          Av = __fma_rn(c.am[j], P[j], Av);
+          if (KIND == 1) Bv = __fma_rn(c.bm[j], P[j], Bv);
         }
-        Rg[(int64_t)j * stride] = R[j];
-        Pg[(int64_t)j * stride] = P[j];
       }
   } else {
-    // large mode counts: several passes over the SoA arrays
-    d0 = decomp_g(M, Rg, stride, n);
-    const double sab = 0.5 * (sigma(al) + sigma(be));
-    const double c0 = DIA ? -1.0 : d0.c2, s0 = DIA ? 0.0 : d0.s2;
-    for (int j = 0; j < n; ++j) {
+    for (int j = 0; j < c.n; ++j) {
       const int64_t o = (int64_t)j * stride;
-      const double x = Rg[o];
-      double p = Pg[o];
-      p += 0.5 * dt * (-M->k[j] * x - (M->s[j] + sab * (M->a[j] * c0 + M->b[j] * s0)));
-      Pg[o] = p;
-      Rg[o] = x + dt * p / M->mass[j];
+      double x = R[o];
+      double p = kick64<KIND, DIA>(c.hk[j], c.hs[j], c.a[j], c.b[j], x, P[o], hu, hv);
+      x = __fma_rn(c.dtm[j], p, x);
+      d.a = __fma_rn(c.a[j], x, d.a);
+      if (KIND == 1) d.b = __fma_rn(c.b[j], x, d.b);
+      R[o] = x;
+      // (the diabatic force does not wait for the decomposition: one pass)
+      P[o] = DIA ? kick64<KIND, DIA>(c.hk[j], c.hs[j], c.a[j], c.b[j], x, p, hu, hv) : p;
     }
-    d1 = decomp_g(M, Rg, stride, n);
-    const double c1 = DIA ? -1.0 : d1.c2, s1 = DIA ? 0.0 : d1.s2;
-    for (int j = 0; j < n; ++j) {
-      const int64_t o = (int64_t)j * stride;
-      const double x = Rg[o];
-      double p = Pg[o];
-      p += 0.5 * dt * (-M->k[j] * x - (M->s[j] + sab * (M->a[j] * c1 + M->b[j] * s1)));
-      Pg[o] = p;
-      if (!DIA) {
-        Av += M->a[j] * (p / M->mass[j]);
-        Bv += M->b[j] * (p / M->mass[j]);
+    decompose64<KIND, DIA>(d);
+    if (!DIA) {
+      const double hu2 = __dmul_rn(hsab, d.c2);
+      const double hv2 = KIND == 1 ? __dmul_rn(hsab, d.s2) : 0.0;
+      for (int j = 0; j < c.n; ++j) {
+        const int64_t o = (int64_t)j * stride;
+        const double p = kick64<KIND, DIA>(c.hk[j], c.hs[j], c.a[j], c.b[j], R[o], P[o], hu2, hv2);
+        Av = __fma_rn(c.am[j], p, Av);
+        if (KIND == 1) Bv = __fma_rn(c.bm[j], p, Bv);
+        P[o] = p;
       }
     }
   }
+  deg |= d.deg;
+  // phase: hbar w_ab = e_a - e_b = (sig_a - sig_b) r; diabatic V_aa - V_bb =
+  // -(sig_a - sig_b) a
+  phi = __fma_rn(DIA ? -wab : wab, __dadd_rn(w0, DIA ? d.a : d.r), phi);
+  // both events have |A_e| = |A|: A = dt g with the coupling contracted with P/M,
+  // g = (a Bv - b Av) / (2 r^2), or c = V_01 dt / hbar (diabatic)
+  double A;
+  if (DIA) A = __dmul_rn(c.cg, d.b);
+  else if (KIND == 1) A = __dmul_rn(__dmul_rn(c.cg, __fma_rn(d.a, Bv, -__dmul_rn(d.b, Av))), d.ir2);
+  else A = __dmul_rn(__dmul_rn(c.cg, Av), d.ir2);
+  // p = min(kappa |A|, p_max) quantised to T = floor(p 2^24); scaling two equal
+  // thresholds down to a sum of at most Tmax in exact integers gives
+  // min(T, floor(Tmax / 2)) (the conversion saturates, and takes 0 for NaN)
+  const uint32_t T = min(__double2uint_rz(__dmul_rn(c.kamp, fabs(A))), c.tmax2);
   Step64 o;
-  o.deg = false;
-  double A1, A2;
-  if (DIA) {
-    // phase: V_aa - V_bb = (d_a - d_b) a = -(sig_a - sig_b) a
-    const double w0 = -(sigma(al) - sigma(be)) * d0.a / M->hbar;
-    const double w1 = -(sigma(al) - sigma(be)) * d1.a / M->hbar;
-    phi += 0.5 * dt * (w0 + w1);
-    // both events have the real factor c = V_01 dt / hbar = b(R_{n+1}) dt / hbar
-    A1 = d1.b * dt / M->hbar;
-    A2 = A1;
-  } else {
-    if (2.0 * d0.r < kDegTol || 2.0 * d1.r < kDegTol) o.deg = true;
-    // phase: hbar w_ab = e_a - e_b = (sig_a - sig_b) r
-    const double w0 = (sigma(al) - sigma(be)) * d0.r / M->hbar;
-    const double w1 = (sigma(al) - sigma(be)) * d1.r / M->hbar;
-    phi += 0.5 * dt * (w0 + w1);
-    // coupling contracted with P/M: g = sum_j (P_j/M_j) d_01,j, d_01,j = (a b_j - b a_j)/(2 r^2)
-    double g = 0.0;
-    if (2.0 * d1.r >= kDegTol) g = (d1.a * Bv - d1.b * Av) / (2.0 * d1.r * d1.r);
-    // events: (first index flips) then (second index flips)
-    A1 = (al == 0) ? dt * g : -(dt * g);
-    A2 = (be == 0) ? dt * g : -(dt * g);
-  }
-  // probabilities min(kappa |A_e|, p_max) quantised to 24-bit thresholds, then
-  // scaled down together in exact integer arithmetic when their sum exceeds Tmax
-  const double p1 = fmin(M->hop_scale * fabs(A1), M->p_max);
-  const double p2 = fmin(M->hop_scale * fabs(A2), M->p_max);
-  uint64_t T1 = (uint64_t)floor(p1 * kP24), T2 = (uint64_t)floor(p2 * kP24);
-  const uint64_t Tmax = (uint64_t)floor(M->p_max * kP24);
-  if (T1 + T2 > Tmax) {
-    const uint64_t sT = T1 + T2;
-    T1 = T1 * Tmax / sT;
-    T2 = T2 * Tmax / sT;
-  }
-  const u4 wd = philox_draw(seed, (uint32_t)(step >> 2), stream, kPurposeHop);
-  const uint32_t y = word_of(wd, (int)(step & 3)) >> 8;
-  if ((uint64_t)y < T1) {  // diabatic: amplitude -i c
-    o.ev = 1;
-    o.num = A1;
-    o.den = (double)T1 / kP24;
-    o.dq = 3;
-  } else if ((uint64_t)y < T1 + T2) {  // diabatic: amplitude +i c
-    o.ev = 2;
-    o.num = A2;
-    o.den = (double)T2 / kP24;
-    o.dq = 1;
-  } else {
-    o.ev = 0;
-    o.num = 1.0;
-    o.den = 1.0 - (double)(T1 + T2) / kP24;
-    o.dq = 0;
-  }
-  if (!DIA) o.dq = 0;
+  o.ev = y < T ? 1 : (y < 2u * T ? 2 : 0);
+  o.dq = (DIA && o.ev) ? (o.ev == 1 ? 3 : 1) : 0;  // amplitudes -i c and +i c
+  const uint32_t iden = o.ev ? T : 16777216u - 2u * T;
+  // A_1 = -sig_a dt g, A_2 = -sig_b dt g (index 0 is sigma = -1)
+  const bool neg = !DIA && (o.ev == 1 ? al : be);
+  const double num = o.ev ? __dmul_rn(neg ? -A : A, kP24) : kP24;
+  o.factor = __dmul_rn(num, rcp_int(int_double(iden), iden));
   return o;
+}
+
+// Loads a walker's modes (NP > 0) and evaluates the decomposition at its R,
+// with the step's operations in its order.
+template <int NP, int NC, int KIND, bool DIA>
+__device__ __forceinline__ void walker_load_f64(const Coef64<NC>& c, const double* Rg,
+                                                const double* Pg, int64_t stride, double* R,
+                                                double* P, Dec64& d) {
+  d.a = c.a0;
+  d.b = c.b0;
+  if constexpr (NP > 0) {
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const bool on = j < c.n;
+      R[j] = on ? Rg[(int64_t)j * stride] : 0.0;
+      P[j] = on ? Pg[(int64_t)j * stride] : 0.0;
+    }
+#pragma unroll
+    for (int j = 0; j < NP; ++j)
+      if (NP <= 4 || j < c.n) {
+        d.a = __fma_rn(c.a[j], R[j], d.a);
+        if (KIND == 1) d.b = __fma_rn(c.b[j], R[j], d.b);
+      }
+  } else {
+    for (int j = 0; j < c.n; ++j) {
+      const double x = Rg[(int64_t)j * stride];
+      d.a = __fma_rn(c.a[j], x, d.a);
+      if (KIND == 1) d.b = __fma_rn(c.b[j], x, d.b);
+    }
+  }
+  decompose64<KIND, DIA>(d);
+}
+
+template <int NP>
+__device__ __forceinline__ void walker_store_f64(int n, const double* R, const double* P,
+                                                 double* Rg, double* Pg, int64_t stride) {
+#pragma unroll
+  for (int j = 0; j < NP; ++j)
+    if (j < n) {
+      Rg[(int64_t)j * stride] = R[j];
+      Pg[(int64_t)j * stride] = P[j];
+    }
+}
+
+// Not finite, by the exponent bits.
+__device__ __forceinline__ bool nonfinite64(double x) {
+  return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000;
+}
+
+// Calls f(NP, NC, KIND, DIA as integral constants) for a model: modes in
+// registers up to 16, beyond in memory.
+template <typename F>
+inline void dispatch_f64(const DevModel& h, F&& f) {
+  auto np = [&](auto NP) {
+    constexpr int np_ = decltype(NP)::value;
+    std::integral_constant<int, (np_ > 0 ? np_ : kMaxN)> NC;
+    const std::integral_constant<int, 0> k0{};
+    const std::integral_constant<int, 1> k1{};
+    if (h.repr == QCL_REPR_DIABATIC)
+      h.kind == 0 ? f(NP, NC, k0, std::true_type{}) : f(NP, NC, k1, std::true_type{});
+    else
+      h.kind == 0 ? f(NP, NC, k0, std::false_type{}) : f(NP, NC, k1, std::false_type{});
+  };
+  if (h.n <= 1) np(std::integral_constant<int, 1>{});
+  else if (h.n <= 2) np(std::integral_constant<int, 2>{});
+  else if (h.n <= 3) np(std::integral_constant<int, 3>{});
+  else if (h.n <= 4) np(std::integral_constant<int, 4>{});
+  else if (h.n <= 8) np(std::integral_constant<int, 8>{});
+  else if (h.n <= 16) np(std::integral_constant<int, 16>{});
+  else np(std::integral_constant<int, 0>{});
 }
 
 // The 16 observable contributions of one walker and their squares (v[16..31]):

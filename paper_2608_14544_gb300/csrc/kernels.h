@@ -305,9 +305,8 @@ struct SpawnLayout {
 void launch_spawn_sample(const DevModel* dm, const SampleParams& sp, int64_t capacity, void* buf,
                          cudaStream_t st);
 // One spawning step (step kernel, scan, scatter) from set step & 1 to the other.
-void launch_spawn_step(const DevModel* dm, int repr, void* buf, int64_t capacity, int n,
-                       int64_t n0, int64_t step0, int64_t step, double dt, uint64_t seed,
-                       cudaStream_t st);
+void launch_spawn_step(const DevModel& host, void* buf, int64_t capacity, int64_t n0,
+                       int64_t step0, int64_t step, double dt, uint64_t seed, cudaStream_t st);
 // Family sums of the current set (set) into per-tile partials (tiles of 256
 // families).
 void launch_spawn_observe(const DevModel* dm, const void* buf, int64_t capacity, int n, int64_t n0,
@@ -352,8 +351,9 @@ void launches_add(int64_t k);
 int64_t launches_read(bool reset);
 
 void launch_sample_f64(const DevModel* dm, const SampleParams& sp, void* buf, cudaStream_t st);
-void launch_step_f64(const DevModel* dm, int repr, void* buf, int64_t nt, int n, int64_t step0,
-                     int64_t step, double dt, uint64_t seed, uint64_t traj_off, cudaStream_t st);
+// Steps [step, step + len) of a two-state ensemble (one launch).
+void launch_steps_f64(const DevModel& host, void* buf, int64_t nt, int64_t step0, int64_t step,
+                      int32_t len, double dt, uint64_t seed, uint64_t traj_off, cudaStream_t st);
 void launch_observe_f64(const DevModel* dm, const void* buf, int64_t nt, int n, double* part,
                         cudaStream_t st);
 

@@ -1,6 +1,7 @@
 // qcl_api.cu -- host implementation of the C ABI declared in include/qcl.h:
 // argument validation, buffer sizing, model constants, and the launch
 // sequences of the FP64 comparator and the FP32-bulk persistent path.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstddef>
@@ -493,15 +494,21 @@ qcl_status qcl_propagate(const qcl_model* model, const qcl_ensemble_desc* ens, v
       launch_fold(part, rows + (size_t)k * q2, fold, OL.n_tiles, q2, 1, s, chunk_row(k));
     };
     if (step0 == 0) observe(0);
-    for (int64_t t = step0; t < step0 + n_steps; ++t) {
+    const int64_t end = step0 + n_steps;
+    for (int64_t t = step0; t < end;) {
+      // two states: up to the next output time in one launch, at most 256 steps
+      // (a launch of 1e7 walkers then stays below a second); more states: one step
+      int64_t len = 1;
+      if (ns == 2) len = std::min<int64_t>(std::min<int64_t>(end, (t / out_stride + 1) * out_stride) - t, 256);
       {
         TimedLaunch tl(1, s);
         if (ns == 2)
-          launch_step_f64(model->dev, model->host.repr, ens_buf, nt, model->n, step0, t, dt, ens->seed, ens->traj_id_offset, s);
+          launch_steps_f64(model->host, ens_buf, nt, step0, t, (int32_t)len, dt, ens->seed, ens->traj_id_offset, s);
         else
           launch_stepN_f64(model->dev, model->host.repr, ns, ens_buf, nt, model->n, step0, t, dt, ens->seed, ens->traj_id_offset, s);
       }
-      if ((t + 1) % out_stride == 0) observe((t + 1) / out_stride);
+      t += len;
+      if (t % out_stride == 0) observe(t / out_stride);
     }
     st = check_launch("FP64 step");
     if (st) return st;
@@ -1002,7 +1009,7 @@ qcl_status qcl_spawn_propagate(const qcl_model* model, const qcl_ensemble_desc* 
       else if (model->ns > 2)
         launch_spawnN_step(model->dev, model->ns, buf, capacity, model->n, n0, step0, t, dt, ens->seed, s);
       else
-        launch_spawn_step(model->dev, model->host.repr, buf, capacity, model->n, n0, step0, t, dt, ens->seed, s);
+        launch_spawn_step(model->host, buf, capacity, n0, step0, t, dt, ens->seed, s);
     }
     if ((t + 1) % out_stride == 0) observe(rows + (size_t)((t + 1) / out_stride) * q2, t + 1);
   }

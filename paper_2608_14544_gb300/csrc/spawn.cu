@@ -83,11 +83,11 @@ __global__ void __launch_bounds__(256) k_spawn_sample(const DevModel* __restrict
 // Step of every live walker of set `src` (in place); the children's weights
 // and pair words go to the per-parent staging arrays, each block's child count
 // to bsum.
-template <int NP, bool DIA>
-__global__ void __launch_bounds__(256) k_spawn_step(const DevModel* __restrict__ M, void* buf,
-                                                    int64_t cap, int n, int64_t n0, int64_t step0,
-                                                    int64_t step, double dt, uint64_t seed) {
-  const SpawnLayout L = SpawnLayout::make(cap, n, n0, QCL_PREC_FP64);
+template <int NP, int NC, int KIND, bool DIA>
+__global__ void __launch_bounds__(256) k_spawn_step(const Coef64<NC> c, void* buf, int64_t cap,
+                                                    int64_t n0, int64_t step0, int64_t step,
+                                                    uint64_t seed) {
+  const SpawnLayout L = SpawnLayout::make(cap, c.n, n0, QCL_PREC_FP64);
   EnsHeader* hdr = (EnsHeader*)buf;
   const int src = (int)(step & 1);
   const int64_t n_live = spawn_header(buf)->n_live[src];
@@ -107,8 +107,15 @@ __global__ void __launch_bounds__(256) k_spawn_step(const DevModel* __restrict__
       const int al = ab & 0xf, be = (ab >> 8) & 0xf, q = (ab >> 4) & 3;
       double phi = w.phi[i];
       const double m = w.m[i];
-      const Step64 o = walker_step_f64<NP, DIA>(M, w.R + i, w.P + i, cap, n, al, be, phi, dt,
-                                                seed, w.id[i], step);
+      double R[NP > 0 ? NP : 1], P[NP > 0 ? NP : 1];
+      Dec64 d;
+      walker_load_f64<NP, NC, KIND, DIA>(c, w.R + i, w.P + i, cap, R, P, d);
+      const u4 wd = philox_draw(seed, (uint32_t)(step >> 2), w.id[i], kPurposeHop);
+      bool deg;
+      const Step64 o = walker_step_f64<NP, NC, KIND, DIA>(
+          c, NP > 0 ? R : w.R + i, NP > 0 ? P : w.P + i, cap, d, al, be, phi,
+          word_of(wd, (int)(step & 3)) >> 8, deg);
+      walker_store_f64<NP>(c.n, R, P, w.R + i, w.P + i, cap);
       w.phi[i] = phi;
       flag = o.ev > 0;
       double* cm = (double*)((char*)buf + L.cm);
@@ -116,7 +123,7 @@ __global__ void __launch_bounds__(256) k_spawn_step(const DevModel* __restrict__
       uint8_t* fl = (uint8_t*)((char*)buf + L.flag);
       fl[i] = (uint8_t)flag;
       if (flag) {
-        const double mc = m * o.num / o.den;
+        const double mc = __dmul_rn(m, o.factor);
         cm[i] = mc;
         cab[i] = (uint16_t)((al ^ (o.ev == 1)) | (((q + o.dq) & 3) << 4) | ((be ^ (o.ev == 2)) << 8));
         if (!isfinite(mc)) {
@@ -124,7 +131,7 @@ __global__ void __launch_bounds__(256) k_spawn_step(const DevModel* __restrict__
           atomicOr(&hdr->flags, QCL_FLAG_NONFINITE);
         }
       }
-      if (o.deg) {
+      if (deg) {
         atomicAdd(&hdr->n_degenerate, 1ull);
         atomicOr(&hdr->flags, QCL_FLAG_DEGENERATE);
       }
@@ -324,23 +331,17 @@ void launch_spawn_sample(const DevModel* dm, const SampleParams& sp, int64_t cap
   launches_add(1);
 }
 
-void launch_spawn_step(const DevModel* dm, int repr, void* buf, int64_t capacity, int n,
-                       int64_t n0, int64_t step0, int64_t step, double dt, uint64_t seed,
-                       cudaStream_t st) {
+void launch_spawn_step(const DevModel& host, void* buf, int64_t capacity, int64_t n0,
+                       int64_t step0, int64_t step, double dt, uint64_t seed, cudaStream_t st) {
   const unsigned nb = spawn_grid(capacity);
-  const bool dia = repr == QCL_REPR_DIABATIC;
-#define QCL_SPAWN_STEP(NP)                                                                   \
-  (dia ? k_spawn_step<NP, true><<<nb, 256, 0, st>>>(dm, buf, capacity, n, n0, step0, step, dt, seed) \
-       : k_spawn_step<NP, false><<<nb, 256, 0, st>>>(dm, buf, capacity, n, n0, step0, step, dt, seed))
-  if (n <= 1)
-    QCL_SPAWN_STEP(1);
-  else if (n <= 4)
-    QCL_SPAWN_STEP(4);
-  else if (n <= 16)
-    QCL_SPAWN_STEP(16);
-  else
-    QCL_SPAWN_STEP(0);
-#undef QCL_SPAWN_STEP
+  const int n = host.n;
+  dispatch_f64(host, [&](auto NP, auto NC, auto KIND, auto DIA) {
+    constexpr int nc = decltype(NC)::value;
+    Coef64<nc> c;
+    make_coef64<nc>(host, dt, c);
+    k_spawn_step<decltype(NP)::value, nc, decltype(KIND)::value, decltype(DIA)::value>
+        <<<nb, 256, 0, st>>>(c, buf, capacity, n0, step0, step, seed);
+  });
   k_spawn_scan<<<1, 1024, 0, st>>>(buf, capacity, n, n0, QCL_PREC_FP64, 2, step0, step);
   k_spawn_scatter<<<nb, 256, 0, st>>>(buf, capacity, n, n0, step0, step, seed);
   launches_add(3);
