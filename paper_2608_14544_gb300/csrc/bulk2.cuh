@@ -67,12 +67,6 @@ __device__ __forceinline__ void renorm(f2& m, int& e) {
 using namespace b2;
 
 // ------------------------------------------------------- persistent step --
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
 // Row stride (floats) of the observation rows in shared memory: 16-byte
 // aligned rows that a warp writes with 128-bit stores (the 8 threads of a
 // quarter warp start 4 banks apart) and reads with 128-bit loads (a quarter
@@ -87,7 +81,7 @@ template <typename V>
 struct ScalV {
   PairV<V> m;
   typename Lanes<V>::I mexp;
-  typename Lanes<V>::I q;  // quarter turns of the weight (diabatic representation)
+  typename Lanes<V>::I q;  // quarter turns of the weight, mod 4 (diabatic representation)
   PairV<V> ph;
   V sa, sb;                // sigma of the index pair: -1 lower, +1 upper adiabatic state
   V A, B;                  // a(R), b(R)
@@ -144,7 +138,7 @@ template <bool S2 = true, typename V>
 __device__ __forceinline__ void closed_form(ScalV<V>& z) {
   z.r2 = vfma(z.A, z.A, vmul(z.B, z.B));
 #pragma unroll
-  for (int l = 0; l < Lanes<V>::W; ++l) ln(z.ir, l) = rsqrtf(fmaxf(ln(z.r2, l), 0x1p-126f));
+  for (int l = 0; l < Lanes<V>::W; ++l) ln(z.ir, l) = rsqrt_normal(fmaxf(ln(z.r2, l), 0x1p-126f));
   z.r = vmul(z.r2, z.ir);
   z.c2 = vmul(z.A, z.ir);
   if (S2) z.s2 = vmul(z.B, z.ir);
@@ -165,7 +159,7 @@ __device__ __forceinline__ void weight_range(ScalV<V>& z, int l) {
   }
 }
 
-// m *= num / den (den an integer below 2^25, so exact in FP32) as a
+// m *= num / den (den an integer of at most 2^24, exact in FP32) as a
 // compensated quotient: rcp.approx, one exact FMA residual, and the product
 // with the error terms collected in lo, then (CHECK) the range check.  The
 // persistent two-state kernels pass CHECK = false and check the range where the
@@ -178,24 +172,61 @@ __device__ __forceinline__ void weight_range(ScalV<V>& z, int l) {
 // |A_e| / p_e ~ 2 |A_e| / p_max, grow with the data; four of them beyond 2^23
 // overflow hi, which the store flags as non-finite.
 template <bool CHECK = true, typename V>
-__device__ __forceinline__ void weight_factor(ScalV<V>& z, V num, const typename Lanes<V>::U& iden) {
-  V den, rd;
+__device__ __forceinline__ void weight_factor(ScalV<V>& z, V num, V den) {
+  V rd;
 #pragma unroll
-  for (int l = 0; l < Lanes<V>::W; ++l) {
-    ln(den, l) = __uint2float_rn(ln(iden, l));
-    ln(rd, l) = rcp_approx(ln(den, l));
-  }
+  for (int l = 0; l < Lanes<V>::W; ++l) ln(rd, l) = rcp_approx(ln(den, l));
   const V q0 = vmul(num, rd);
   // num - q0 den = fma(q0, -den, num), exactly as fma(-q0, den, num)
-  const V q1 = vmul(vfma(q0, vmul(den, splat<V>(-1.0f)), num), rd);
+  const V q1 = vmul(vfma(q0, vneg(den), num), rd);
   const V p = vmul(z.m.hi, q0);
-  V e = vfma(z.m.hi, q0, vmul(p, splat<V>(-1.0f)));
+  V e = vfma(z.m.hi, q0, vneg(p));
   e = vfma(z.m.hi, q1, e);
   z.m = {p, vfma(z.m.lo, q0, e)};
   if (CHECK) {
 #pragma unroll
     for (int l = 0; l < Lanes<V>::W; ++l) weight_range(z, l);
   }
+}
+
+// The transition test of a walker's two equally likely events against the
+// 24-bit number y of its hop word: the threshold T = min(floor(|t|), thalf) with
+// t = kappa |A| 2^24 and thalf = floor(Tmax / 2) < 2^23, event 1 where y < T,
+// event 2 where T <= y < 2T, and the weight's divisor den (T on an event,
+// 2^24 - 2T otherwise).  T is taken as the low bits of 2^23 + |t| rounded towards
+// zero, so that neither a float-to-integer conversion nor its reverse is needed:
+// the sum's bits are 0x4B000000 + T and compare as integers with 0x4B000000 + y.
+// (An amplitude that is not a number takes T = thalf; its walker is reported
+// non-finite.)
+template <typename V>
+struct HopTest {
+  bool hop1[Lanes<V>::W], hop2[Lanes<V>::W], hop[Lanes<V>::W];
+  V den;
+};
+__device__ __forceinline__ float vadd_rz(float a, float b) { return __fadd_rz(a, b); }
+__device__ __forceinline__ float2 vadd_rz(float2 a, float2 b) { return __fadd2_rz(a, b); }
+
+template <typename V>
+__device__ __forceinline__ HopTest<V> hop_test(V t, const typename Lanes<V>::U& word,
+                                               const BulkParams& bp) {
+  constexpr int W = Lanes<V>::W;
+  HopTest<V> h;
+  V a;
+#pragma unroll
+  for (int l = 0; l < W; ++l) ln(a, l) = fminf(fabsf(ln(t, l)), bp.thalf);
+  a = vadd_rz(a, splat<V>(0x1p23f));
+  const V T = vadd(a, splat<V>(-0x1p23f));
+  const V stay = vfma(T, splat<V>(-2.0f), splat<V>(0x1p24f));
+#pragma unroll
+  for (int l = 0; l < W; ++l) {
+    const uint32_t y = __byte_perm(ln(word, l), 0x4Bu, 0x4321);  // 0x4B000000 + (word >> 8)
+    const uint32_t u = __float_as_uint(ln(a, l));
+    h.hop1[l] = y < u;
+    h.hop[l] = y < u + u - 0x4B000000u;
+    h.hop2[l] = h.hop[l] && !h.hop1[l];
+    ln(h.den, l) = h.hop[l] ? ln(T, l) : ln(stay, l);
+  }
+  return h;
 }
 
 // Phase (trapezoid) and transition of one step, given the decomposition at
@@ -215,16 +246,17 @@ __device__ __forceinline__ void phase_and_transition(ScalV<V>& z, V r_old, V Av,
   // phase: dt/2 (w_ab(R_n) + w_ab(R_{n+1})), hbar w_ab = (sig_a - sig_b) r, added
   // to the low word of the pair (at most four increments and their rounding
   // errors until block_end folds it into hi)
-  // LANE_PHASE: per lane with the scalar round-to-nearest operations.  Measured
-  // on GB300: in the branch-free step (CHECK = false) the packed form of this one
-  // update gave results one ulp apart between one and two walkers per thread,
-  // while the per-lane form keeps both bit for bit (and equal to the packed form
-  // in the step with the range check).
+  // LANE_PHASE: r_n + r_{n+1} per lane with the scalar round-to-nearest
+  // operation.  Measured on GB300: in the branch-free step (CHECK = false) the
+  // packed form of this sum gave results one ulp apart between one and two
+  // walkers per thread, while the per-lane form keeps both bit for bit (and equal
+  // to the packed form in the step with the range check).
   if (WEIGHT && LANE_PHASE) {
+    // (the pair's factor is an exact power-of-two multiple: packed)
+    V rr;
 #pragma unroll
-    for (int l = 0; l < W; ++l)
-      ln(z.ph.lo, l) = __fmaf_rn(__fmul_rn(bp.hdt_hbar, __fsub_rn(ln(z.sa, l), ln(z.sb, l))),
-                                 __fadd_rn(ln(r_old, l), ln(z.r, l)), ln(z.ph.lo, l));
+    for (int l = 0; l < W; ++l) ln(rr, l) = __fadd_rn(ln(r_old, l), ln(z.r, l));
+    z.ph.lo = vfma(vmul(splat<V>(bp.hdt_hbar), vsub(z.sa, z.sb)), rr, z.ph.lo);
   } else if (WEIGHT) {
     z.ph.lo = vfma(vmul(splat<V>(bp.hdt_hbar), vsub(z.sa, z.sb)), vadd(r_old, z.r), z.ph.lo);
   }
@@ -237,9 +269,7 @@ __device__ __forceinline__ void phase_and_transition(ScalV<V>& z, V r_old, V Av,
   // both events have |A_e| = dt |g|: p = min(kappa dt |g|, p_max) quantised to
   // 24-bit thresholds T = floor(p 2^24); when 2T exceeds Tmax = floor(p_max 2^24)
   // the integer rescale floor(T Tmax / 2T) gives floor(Tmax / 2), so
-  // T = min(floor(kappa dt |g| 2^24), floor(Tmax / 2)) (the conversion saturates)
-  typename Lanes<V>::U T, iden;
-  bool hop1[W], hop2[W], hop[W];
+  // T = min(floor(kappa dt |g| 2^24), floor(Tmax / 2))
   if (KIND == 1) {  // (the spin-boson form runs only where r^2 >= b0^2 excludes degeneracy)
 #pragma unroll
     for (int l = 0; l < W; ++l) {
@@ -248,31 +278,22 @@ __device__ __forceinline__ void phase_and_transition(ScalV<V>& z, V r_old, V Av,
       ln(g, l) = degen ? 0.0f : ln(g, l);
     }
   }
-  const V t = vmul(splat<V>(bp.kamp * kP24f), g);
+  const HopTest<V> h = hop_test(vmul(splat<V>(bp.kamp * kP24f), g), word, bp);
   // weight factor: A_e / p_hat on a hop (A_1 = -sig_a dt g, A_2 = -sig_b dt g),
   // 1 / (1 - sum p_hat) otherwise
   const V dtgn = vmul(splat<V>(-(bp.amp * kP24f)), g);
   V sel;
 #pragma unroll
-  for (int l = 0; l < W; ++l) {
-    ln(T, l) = min(__float2uint_rz(fabsf(ln(t, l))), bp.tmax >> 1);
-    const uint32_t y = ln(word, l) >> 8;
-    hop1[l] = y < ln(T, l);
-    hop[l] = y < 2u * ln(T, l);
-    hop2[l] = hop[l] && !hop1[l];
-    ln(sel, l) = hop1[l] ? ln(z.sa, l) : ln(z.sb, l);
-    ln(iden, l) = hop[l] ? ln(T, l) : 16777216u - 2u * ln(T, l);
-  }
+  for (int l = 0; l < W; ++l) ln(sel, l) = h.hop1[l] ? ln(z.sa, l) : ln(z.sb, l);
   V num = vmul(sel, dtgn);
-  const V nsa = vmul(z.sa, splat<V>(-1.0f)), nsb = vmul(z.sb, splat<V>(-1.0f));
 #pragma unroll
   for (int l = 0; l < W; ++l) {
-    ln(num, l) = hop[l] ? ln(num, l) : kP24f;
-    ln(z.sa, l) = hop1[l] ? ln(nsa, l) : ln(z.sa, l);
-    ln(z.sb, l) = hop2[l] ? ln(nsb, l) : ln(z.sb, l);
+    ln(num, l) = h.hop[l] ? ln(num, l) : kP24f;
+    ln(z.sa, l) = h.hop1[l] ? -ln(z.sa, l) : ln(z.sa, l);
+    ln(z.sb, l) = h.hop2[l] ? -ln(z.sb, l) : ln(z.sb, l);
   }
   // (sigmas flipped after the weight factor has taken the pre-hop sigma in sel)
-  if (WEIGHT) weight_factor<CHECK>(z, num, iden);
+  if (WEIGHT) weight_factor<CHECK>(z, num, h.den);
 }
 
 // Diabatic representation: phase with hbar w_ab = V_aa - V_bb = -(sig_a - sig_b)
@@ -286,31 +307,24 @@ __device__ __forceinline__ void dia_phase_and_transition(ScalV<V>& z, V a_old, V
                                                          const typename Lanes<V>::U& word,
                                                          const BulkParams& bp) {
   constexpr int W = Lanes<V>::W;
+  V aa;
 #pragma unroll
   for (int l = 0; l < W; ++l)  // (per lane, as in phase_and_transition)
-    ln(z.ph.lo, l) = __fmaf_rn(__fmul_rn(bp.hdt_hbar, __fsub_rn(ln(z.sb, l), ln(z.sa, l))),
-                               __fadd_rn(ln(a_old, l), ln(z.A, l)), ln(z.ph.lo, l));
-  const V t = vmul(splat<V>(bp.kamp * kP24f), Bc);
+    ln(aa, l) = __fadd_rn(ln(a_old, l), ln(z.A, l));
+  z.ph.lo = vfma(vmul(splat<V>(bp.hdt_hbar), vsub(z.sb, z.sa)), aa, z.ph.lo);
+  const HopTest<V> h = hop_test(vmul(splat<V>(bp.kamp * kP24f), Bc), word, bp);
   V num = vmul(splat<V>(bp.amp * kP24f), Bc);
-  typename Lanes<V>::U iden;
-  bool hop1[W], hop2[W], hop[W];
+#pragma unroll
+  for (int l = 0; l < W; ++l) ln(num, l) = h.hop[l] ? ln(num, l) : kP24f;
+  weight_factor<CHECK>(z, num, h.den);
 #pragma unroll
   for (int l = 0; l < W; ++l) {
-    const uint32_t T = min(__float2uint_rz(fabsf(ln(t, l))), bp.tmax >> 1);
-    const uint32_t y = ln(word, l) >> 8;
-    hop1[l] = y < T;
-    hop[l] = y < 2u * T;
-    hop2[l] = hop[l] && !hop1[l];
-    ln(num, l) = hop[l] ? ln(num, l) : kP24f;
-    ln(iden, l) = hop[l] ? T : 16777216u - 2u * T;
-  }
-  weight_factor<CHECK>(z, num, iden);
-  const V nsa = vmul(z.sa, splat<V>(-1.0f)), nsb = vmul(z.sb, splat<V>(-1.0f));
-#pragma unroll
-  for (int l = 0; l < W; ++l) {
-    ln(z.q, l) = (ln(z.q, l) + (hop1[l] ? 3 : (hop2[l] ? 1 : 0))) & 3;
-    ln(z.sa, l) = hop1[l] ? ln(nsa, l) : ln(z.sa, l);
-    ln(z.sb, l) = hop2[l] ? ln(nsb, l) : ln(z.sb, l);
+    // quarter turns, three (that is, one back) or one: counted without the
+    // reduction mod 4, which every reader of q makes
+    if (h.hop1[l]) ln(z.q, l) -= 1;
+    if (h.hop2[l]) ln(z.q, l) += 1;
+    ln(z.sa, l) = h.hop1[l] ? -ln(z.sa, l) : ln(z.sa, l);
+    ln(z.sb, l) = h.hop2[l] ? -ln(z.sb, l) : ln(z.sb, l);
   }
 }
 
@@ -445,7 +459,7 @@ __device__ __forceinline__ bool spawn_transition(Scal& z, float w_old, float Av,
   child = z;
   // adiabatic: A_1 = -sig_a dt g, A_2 = -sig_b dt g; diabatic: both c = b dt / hbar
   const float num = DIA ? fac : -(hop1 ? z.sa : z.sb) * fac;
-  weight_factor(child, num, T);
+  weight_factor(child, num, __uint2float_rn(T));
   child.m = fast_two_sum(child.m.hi, child.m.lo);
   if (hop1) child.sa = -child.sa;
   else child.sb = -child.sb;
@@ -489,7 +503,7 @@ __device__ __forceinline__ Contrib contrib_factors(const Scal& z, float mm) {
   // exact degeneracy (both 0) theta = 0
   const float c2 = (z.c2 == 0.0f && z.s2 == 0.0f) ? 1.0f : z.c2;
   const float t = __fmaf_rn(0.5f, fabsf(c2), 0.5f);
-  const float rt = rsqrtf(t);
+  const float rt = rsqrt_normal(t);
   const float big = t * rt, small = 0.5f * fabsf(z.s2) * rt;
   const bool cpos = c2 >= 0.0f;
   const float c = cpos ? big : small;
@@ -890,7 +904,7 @@ __device__ __forceinline__ void bulk2_tile(const BulkParams& bp, const CF& cf, W
     ws.me[i] = ln(z.mexp, k);
     ws.ph[i] = ph;
     ws.pl[i] = ln(z.ph.lo, k);
-    ws.ab[i] = (uint16_t)((ln(z.sa, k) > 0.0f ? 1 : 0) | (ln(z.q, k) << 4) |
+    ws.ab[i] = (uint16_t)((ln(z.sa, k) > 0.0f ? 1 : 0) | ((ln(z.q, k) & 3) << 4) |
                           ((ln(z.sb, k) > 0.0f ? 1 : 0) << 8));
     if (!isfinite(mh) || !isfinite(ph)) {
       atomicAdd(&ws.hdr->n_nonfinite, 1ull);

@@ -108,6 +108,7 @@ struct BulkParams {
   float kamp;          // hop_scale * amp
   float p_max;
   uint32_t tmax;       // floor(p_max 2^24)
+  float thalf;         // floor(tmax / 2) (below 2^23, so exact)
   float kappa;         // hop_scale
   // sum_j a_j a_j / M_j, sum_j a_j b_j / M_j, sum_j b_j b_j / M_j over the
   // FP32 coefficients (the split kernel's one-exchange coupling sums)
@@ -146,6 +147,7 @@ inline void bulk_model_scalars(BulkParams& bp, const DevModel& h, double dt) {
   bp.kamp = (float)(h.hop_scale * amp);
   bp.p_max = (float)h.p_max;
   bp.tmax = (uint32_t)std::floor(h.p_max * kP24);
+  bp.thalf = (float)(bp.tmax >> 1);
   bp.kappa = (float)h.hop_scale;
   double caa = 0.0, cab = 0.0, cbb = 0.0;
   for (int j = 0; j < h.n; ++j) {

@@ -503,7 +503,7 @@ __device__ __forceinline__ void split_tiles_dia(const BulkParams& bp, const Coef
         ws.me[i] = ln(z.mexp, k);
         ws.ph[i] = ph;
         ws.pl[i] = ln(z.ph.lo, k);
-        ws.ab[i] = (uint16_t)((ln(z.sa, k) > 0.0f ? 1 : 0) | (ln(z.q, k) << 4) |
+        ws.ab[i] = (uint16_t)((ln(z.sa, k) > 0.0f ? 1 : 0) | ((ln(z.q, k) & 3) << 4) |
                               ((ln(z.sb, k) > 0.0f ? 1 : 0) << 8));
         if (!isfinite(mh) || !isfinite(ph)) {
           atomicAdd(&ws.hdr->n_nonfinite, 1ull);

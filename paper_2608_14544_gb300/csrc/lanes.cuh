@@ -45,9 +45,41 @@ template <>
 __device__ __forceinline__ float splat<float>(float c) { return c; }
 template <>
 __device__ __forceinline__ float2 splat<float2>(float c) { return make_float2(c, c); }
+// -a: an operand modifier of the instruction that takes it, packed ones
+// included (measured: a chain of packed FMAs with a negated operand issues one
+// instruction a link, one with a multiplication by -1 two)
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
 // a - b = fma(b, -1, a) exactly (one rounding, as a subtraction)
 template <typename V>
 __device__ __forceinline__ V vsub(V a, V b) { return vfma(b, splat<V>(-1.0f), a); }
+
+// The hardware reciprocal square root, reciprocal and approximate quotient
+// without the library forms' rescaling of subnormal operands (two to five more
+// instructions each): for normal operands and results the same bits as
+// rsqrtf (compared on every positive normal float) and __fdividef (compared on
+// 2^31 random pairs); subnormals count as zero.
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float div_normal(float a, float b) {
+  float r;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+// 1 / d correctly rounded for an integer 1 <= d <= 2^24 (one Newton step on the
+// hardware reciprocal; equal to __frcp_rn at every such d).
+__device__ __forceinline__ float rcp_integer(float d) {
+  const float r = rcp_approx(d);
+  return __fmaf_rn(r, __fmaf_rn(-d, r, 1.0f), r);
+}
 
 // lane l of a value (l a compile-time constant after unrolling)
 __device__ __forceinline__ float& ln(float& v, int) { return v; }
@@ -86,7 +118,7 @@ __device__ __forceinline__ PairV<V> df_add_v(PairV<V> a, V b) {
 template <typename V>
 __device__ __forceinline__ PairV<V> df_mul_v(PairV<V> a, V q0, V q1) {
   const V p = vmul(a.hi, q0);
-  V e = vfma(a.hi, q0, vmul(p, splat<V>(-1.0f)));
+  V e = vfma(a.hi, q0, vneg(p));
   e = vfma(a.hi, q1, e);
   e = vfma(a.lo, q0, e);
   return fast_two_sum_v(p, e);

@@ -224,7 +224,7 @@ __device__ __forceinline__ void jacobi_sweep_warm(V (&A)[NS][NS], V (&U)[NS][NS]
       if (small) {
 #pragma unroll
         for (int l = 0; l < L; ++l) {  // (a zero a_pq gives t = 0, also where d = 0)
-          const float q = __fdividef(ln(apq, l), ln(d, l));
+          const float q = div_normal(ln(apq, l), ln(d, l));
           ln(t, l) = ln(apq, l) == 0.0f ? 0.0f : q;
         }
         sn = t;
@@ -233,21 +233,23 @@ __device__ __forceinline__ void jacobi_sweep_warm(V (&A)[NS][NS], V (&U)[NS][NS]
         const V r2 = vfma(d, d, vmul(twoa, twoa));
 #pragma unroll
         for (int l = 0; l < L; ++l) {
-          // d + sgn(d) sqrt(d^2 + 4 a_pq^2) is never 0 unless a_pq = 0 (then t = 0)
+          // d + sgn(d) sqrt(d^2 + 4 a_pq^2) is never 0 unless a_pq = 0 (then t = 0;
+          // gap and coupling both below 1e-19, thirteen orders under the degeneracy
+          // threshold, also give t = 0)
           const float rl = ln(r2, l);
-          const float den = ln(d, l) + copysignf(rl * rsqrtf(rl), ln(d, l));
-          const float q = __fdividef(ln(twoa, l), den);
+          const float den = ln(d, l) + copysignf(rl * rsqrt_normal(rl), ln(d, l));
+          const float q = div_normal(ln(twoa, l), den);
           ln(t, l) = ln(apq, l) == 0.0f ? 0.0f : q;
         }
         const V tt1 = vfma(t, t, splat<V>(1.0f));
 #pragma unroll
-        for (int l = 0; l < L; ++l) ln(c, l) = rsqrtf(ln(tt1, l));
+        for (int l = 0; l < L; ++l) ln(c, l) = rsqrt_normal(ln(tt1, l));
         sn = vmul(t, c);
       }
 #pragma unroll
       for (int l = 0; l < L; ++l) ln(tm, l) = fmaxf(ln(tm, l), fabsf(ln(t, l)));
-      const V nsn = vmul(sn, splat<V>(-1.0f));
-      A[p][p] = vfma(t, vmul(apq, splat<V>(-1.0f)), A[p][p]);  // a_pp - t a_pq
+      const V nsn = vneg(sn);
+      A[p][p] = vfma(t, vneg(apq), A[p][p]);  // a_pp - t a_pq
       A[q][q] = vfma(t, apq, A[q][q]);
       A[p][q] = splat<V>(0.0f);
 #pragma unroll

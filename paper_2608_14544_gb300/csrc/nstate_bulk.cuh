@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
               // approximate division (the amplitude enters a probability and a
               // weight factor, both far above its 2-ulp error), taken on every
               // slot and discarded by the select (no branch around it)
-              const float qd = __fdividef(ln(h, l), ln(gap, l));
+              const float qd = div_normal(ln(h, l), ln(gap, l));
               ln(vd, l) = (!evl || dg) ? 0.0f : qd;
             }
             A[sl * NS + nu] = vmul(splat<V>(sl == 0 ? -bp.dt : bp.dt), vd);
@@ -701,11 +701,11 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
         const bool hop = hit >= 0;
         ln(num, l) = hop ? Ah * kP24f : kP24f;
         ln(den, l) = __uint2float_rn(hop ? Th : 16777216u - sumT);
-        ln(rd, l) = __frcp_rn(ln(den, l));
+        ln(rd, l) = rcp_integer(ln(den, l));
         hitl[l] = hit;
       }
       const V q0 = vmul(num, rd);
-      const V q1 = vmul(vfma(q0, vmul(den, splat<V>(-1.0f)), num), rd);
+      const V q1 = vmul(vfma(q0, vneg(den), num), rd);
       m = df_mul_v(m, q0, q1);
 #pragma unroll
       for (int l = 0; l < WPT; ++l) {
@@ -1063,7 +1063,7 @@ __global__ void __launch_bounds__(128, (NPL > 8 || NS > 5) ? 2 : 4)
       const bool hop = hit >= 0;
       const float num = hop ? ch * kP24f : kP24f;
       const float den = __uint2float_rn(hop ? Th : 16777216u - sumT);
-      const float rd = __frcp_rn(den);
+      const float rd = rcp_integer(den);
       const float q0 = __fmul_rn(num, rd);
       const float q1 = __fmul_rn(__fmaf_rn(-q0, den, num), rd);
       m = df_mul(m, q0, q1);

@@ -123,7 +123,7 @@ __device__ __forceinline__ T quot(T a, T b) {
 }
 template <>
 __device__ __forceinline__ float quot<float>(float a, float b) {
-  return __fdividef(a, b);
+  return div_normal(a, b);
 }
 
 // (with columns al, be of U already extracted into ua, ub)

@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(256) k_spawnN_step32(const BulkParams bp, cons
             const bool evl = (sl == 0) ? (nu != al) : (nu != be);
             const bool dg = evl && fabsf(gp) < kDegTolF;
             deg |= dg;
-            const float qd = __fdividef(h, gp);
+            const float qd = div_normal(h, gp);
             A[sl * NS + nu] = __fmul_rn(sl == 0 ? -bp.dt : bp.dt, (!evl || dg) ? 0.0f : qd);
           }
         if (live) {
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(256) k_spawnN_step32(const BulkParams bp, cons
           Th = (k == hit) ? T[k] : Th;
         }
         const float num = Ah * kP24f, den = __uint2float_rn(Th);
-        const float rd = __frcp_rn(den);
+        const float rd = rcp_integer(den);
         const float q0 = __fmul_rn(num, rd);
         const float q1 = __fmul_rn(__fmaf_rn(-q0, den, num), rd);
         f2 cm = df_mul({s.mh[i], s.ml[i]}, q0, q1);
