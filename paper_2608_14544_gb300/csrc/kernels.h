@@ -195,6 +195,14 @@ __device__ __forceinline__ double coef_dt(const CoefN& c) {
   return __hiloint2double((int)c.dt_w[1], (int)c.dt_w[0]);
 }
 
+// The model on the host and dt, for launchers that build larger coefficient
+// blocks than CoefN.
+struct ModeHost {
+  const DevModel* h;
+  const double* K;  // [n][N_s * N_s]
+  double dt;
+};
+
 // One request of a packed launch: a two-state model with at most 8 modes
 // advancing over its own steps [cs, ce) (device table entry).
 constexpr int kMaxPacked = 256;
@@ -410,8 +418,8 @@ void launch_stepN_f64(const DevModel* dm, int repr, int ns, void* buf, int64_t n
                       cudaStream_t st);
 void launch_observeN_f64(const DevModel* dm, int ns, const void* buf, int64_t nt, int n,
                          double* part, cudaStream_t st);
-int launch_bulkN(int ns, const BulkParams& bp, const CoefN& cf, void* buf, double* part,
-                 const LaunchShape& ls, cudaStream_t st);
+int launch_bulkN(int ns, const BulkParams& bp, const CoefN& cf, const ModeHost& mh, void* buf,
+                 double* part, const LaunchShape& ls, cudaStream_t st);
 
 // Folds n_slots output times of per-tile partials into rows; with chunk_out
 // (rows of [n_slots][ceil(n_tiles / 1024)][q2]) the first level's 1024-tile

@@ -10,7 +10,7 @@ namespace qcl {
   void nstate_step64_##k(const DevModel*, int, void*, int64_t, int, int64_t, int64_t, double, \
                          uint64_t, uint64_t, cudaStream_t);                                   \
   void nstate_observe64_##k(const DevModel*, const void*, int64_t, int, double*, cudaStream_t); \
-  int nstate_bulk_##k(const BulkParams&, const CoefN&, void*, double*, int, int, cudaStream_t); \
+  int nstate_bulk_##k(const BulkParams&, const CoefN&, const ModeHost&, void*, double*, int, int, cudaStream_t); \
   void nstate_spawn_sample64_##k(const DevModel*, const SampleParams&, int64_t, void*,        \
                                  cudaStream_t);                                               \
   void nstate_spawn_step64_##k(const DevModel*, void*, int64_t, int, int64_t, int64_t, int64_t, \
@@ -103,8 +103,8 @@ void launch_spawnN_observe32(int ns, const BulkParams& bp, const CoefN& cf, cons
   QCL_NS_SWITCH(ns, nstate_spawn_observe32, bp, cf, buf, capacity, n0, set, part, st);
 }
 
-int launch_bulkN(int ns, const BulkParams& bp, const CoefN& cf, void* buf, double* part,
-                 const LaunchShape& ls, cudaStream_t st) {
+int launch_bulkN(int ns, const BulkParams& bp, const CoefN& cf, const ModeHost& mh, void* buf,
+                 double* part, const LaunchShape& ls, cudaStream_t st) {
   // blocks per SM become a cap on the grid (one walker per thread here)
   static int n_sm = 0;
   if (n_sm == 0) {
@@ -117,12 +117,12 @@ int launch_bulkN(int ns, const BulkParams& bp, const CoefN& cf, void* buf, doubl
     grid_cap = ls.blocks_per_sm * n_sm;
   int g = 0;
   switch (ns) {
-    case 3: g = nstate_bulk_3(bp, cf, buf, part, grid_cap, ls.wpt, st); break;
-    case 4: g = nstate_bulk_4(bp, cf, buf, part, grid_cap, ls.wpt, st); break;
-    case 5: g = nstate_bulk_5(bp, cf, buf, part, grid_cap, ls.wpt, st); break;
-    case 6: g = nstate_bulk_6(bp, cf, buf, part, grid_cap, ls.wpt, st); break;
-    case 7: g = nstate_bulk_7(bp, cf, buf, part, grid_cap, ls.wpt, st); break;
-    case 8: g = nstate_bulk_8(bp, cf, buf, part, grid_cap, ls.wpt, st); break;
+    case 3: g = nstate_bulk_3(bp, cf, mh, buf, part, grid_cap, ls.wpt, st); break;
+    case 4: g = nstate_bulk_4(bp, cf, mh, buf, part, grid_cap, ls.wpt, st); break;
+    case 5: g = nstate_bulk_5(bp, cf, mh, buf, part, grid_cap, ls.wpt, st); break;
+    case 6: g = nstate_bulk_6(bp, cf, mh, buf, part, grid_cap, ls.wpt, st); break;
+    case 7: g = nstate_bulk_7(bp, cf, mh, buf, part, grid_cap, ls.wpt, st); break;
+    case 8: g = nstate_bulk_8(bp, cf, mh, buf, part, grid_cap, ls.wpt, st); break;
     default: break;
   }
   if (g) launches_add(1);

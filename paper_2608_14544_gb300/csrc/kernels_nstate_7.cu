@@ -10,9 +10,9 @@ void nstate_observe64_7(const DevModel* dm, const void* buf, int64_t nt, int n, 
                          cudaStream_t st) {
   NStateOps<7>::observe64(dm, buf, nt, n, part, st);
 }
-int nstate_bulk_7(const BulkParams& bp, const CoefN& cf, void* buf, double* part, int grid_cap,
-                  int wpt, cudaStream_t st) {
-  return NStateOps<7>::bulk(bp, cf, buf, part, grid_cap, wpt, st);
+int nstate_bulk_7(const BulkParams& bp, const CoefN& cf, const ModeHost& mh, void* buf,
+                  double* part, int grid_cap, int wpt, cudaStream_t st) {
+  return NStateOps<7>::bulk(bp, cf, mh, buf, part, grid_cap, wpt, st);
 }
 void nstate_spawn_sample32_7(const SampleN32& sp, int64_t cap, void* buf, cudaStream_t st) {
   NStateOps<7>::spawn_sample32(sp, cap, buf, st);

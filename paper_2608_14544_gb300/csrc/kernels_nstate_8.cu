@@ -10,9 +10,9 @@ void nstate_observe64_8(const DevModel* dm, const void* buf, int64_t nt, int n, 
                          cudaStream_t st) {
   NStateOps<8>::observe64(dm, buf, nt, n, part, st);
 }
-int nstate_bulk_8(const BulkParams& bp, const CoefN& cf, void* buf, double* part, int grid_cap,
-                  int wpt, cudaStream_t st) {
-  return NStateOps<8>::bulk(bp, cf, buf, part, grid_cap, wpt, st);
+int nstate_bulk_8(const BulkParams& bp, const CoefN& cf, const ModeHost& mh, void* buf,
+                  double* part, int grid_cap, int wpt, cudaStream_t st) {
+  return NStateOps<8>::bulk(bp, cf, mh, buf, part, grid_cap, wpt, st);
 }
 void nstate_spawn_sample32_8(const SampleN32& sp, int64_t cap, void* buf, cudaStream_t st) {
   NStateOps<8>::spawn_sample32(sp, cap, buf, st);

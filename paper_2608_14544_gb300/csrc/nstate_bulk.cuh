@@ -211,6 +211,29 @@ __device__ __forceinline__ void mode_row(const float* mt, int j, float (&r)[Mode
   }
 }
 
+// The same rows as a kernel parameter (N_s <= 4, up to NM modes), read as
+// constant-bank operands at warp-uniform addresses.
+template <int NS, int NM>
+struct CoefMem {
+  alignas(16) float row[NM][ModeRow<NS>::CS];
+};
+template <int NS>
+struct CoefMem<NS, 0> {};
+
+// The values of fill_mode_table, on the host.
+template <int NS, int NM>
+inline void make_coef_mem(const ModeHost& mh, int n, CoefMem<NS, NM>& c) {
+  using MR = ModeRow<NS>;
+  for (int j = 0; j < n; ++j) {
+    const double* Kj = mh.K + (size_t)j * NS * NS;
+    for (int a = 0; a < NS; ++a)
+      for (int b = a; b < NS; ++b) c.row[j][tri<NS>(a, b)] = (float)Kj[a * NS + b];
+    c.row[j][MR::HK] = (float)(0.5 * mh.dt * mh.h->k[j]);
+    c.row[j][MR::DTM] = (float)(mh.dt / mh.h->mass[j]);
+    c.row[j][MR::MINV] = (float)(1.0 / mh.h->mass[j]);
+  }
+}
+
 // WPT (1 or 2) tiles of 128 walkers per block, thread t holding walker t of
 // each: with WPT = 2 the two walkers are the lanes of float2 values and their
 // FP32 arithmetic runs as packed FP32x2 instructions (explicit round-to-nearest
@@ -222,11 +245,18 @@ struct BulkNMinBlocks {
       NPL > 8 ? 1 : (WPT == 1 ? (NS <= 4 ? 4 : (NS == 5 ? 3 : 1)) : (NS <= 4 ? 2 : 1));
 };
 
-template <int NS, int NPL, int WPT>
+template <int NS, int NPL, int WPT, int NM = 0, int SM = 0>
 __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
-    k_bulkN(const BulkParams bp, const CoefN cf, void* buf, double* __restrict__ part) {
+    k_bulkN(const BulkParams bp, const CoefN cf, void* buf, double* __restrict__ part,
+            const CoefMem<NS, NM> cm) {
   static_assert(WPT == 1 || WPT == 2, "one or two walkers per thread");
-  // NPL = 0: the modes stay in memory (any mode count, one walker per thread)
+  // NPL = 0: the modes stay in memory (any mode count, one walker per thread).
+  // Measured on the four-state 64-mode model: 6616 instructions a walker-step,
+  // 108 a mode of which 60 are the FMAs; the rest were 64-bit addresses, selects
+  // for lanes past the ensemble and 128-bit loads of the coefficient rows.
+  // Rows as uniform constant operands and R, P at fixed shared-memory offsets
+  // leave 96; two walkers per thread (half the instructions) was no faster: at
+  // 168-226 registers 8-12 warps an SM do not hide the loads.
   constexpr bool MEM = NPL == 0;
   constexpr int NR = MEM ? 1 : NPL;
   static_assert(!MEM || WPT == 1, "modes in memory: one walker per thread");
@@ -240,12 +270,16 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
   __shared__ float obs_rows[TW * 33];
   extern __shared__ float4 mode_tab4[];
   float* const mtab = reinterpret_cast<float*>(mode_tab4);
+  // (SM > 0: P, and with SM = 2 also R, of the block's walkers, row j of the
+  // mode at j * TW)
+  float* const Ps = mtab + threadIdx.x;
+  float* const Rs = Ps + (SM == 2 ? bp.n * TW : 0);
   WN<float> ws = viewN<float>(buf, bp.n_traj, NS, bp.n, QCL_PREC_FP32_BULK);
   if (ws.hdr->step != bp.step0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ws.hdr->flags, QCL_FLAG_STEP_MISMATCH);
     return;
   }
-  if constexpr (MEM) fill_mode_table<NS>(mtab, coef_dm(cf), coef_dt(cf), bp.n);
+  if constexpr (MEM && NM == 0) fill_mode_table<NS>(mtab, coef_dm(cf), coef_dt(cf), bp.n);
   const int64_t nt = bp.n_traj;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned int n_deg = 0;
@@ -371,9 +405,18 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
     // after, so that a batch's loads are not ordered behind the previous
     // mode's stores (lanes past the ensemble load walker 0's values, take
     // zeros as the register form does, and store nothing).
+    // mode jj's coefficients: constant-bank rows, or the shared table
+    auto mrow = [&](int jj, float (&kr)[MR::CS]) {
+      if constexpr (NM > 0) {
+#pragma unroll
+        for (int c = 0; c < MR::CS; ++c) kr[c] = cm.row[jj][c];
+      } else {
+        mode_row<NS>(mtab, jj, kr);
+      }
+    };
     auto mode_a = [&](int jj, const V (&Q)[NTRI], V (&t)[NTRI], V& r, V& p) {
       float kr[MR::CS];
-      mode_row<NS>(mtab, jj, kr);
+      mrow(jj, kr);
       V g = splat<V>(0.0f);
 #pragma unroll
       for (int k = 0; k < NTRI; ++k) g = vfma(splat<V>(kr[k]), Q[k], g);
@@ -384,7 +427,7 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
     };
     auto mode_b = [&](int jj, const V (&Q)[NTRI], V (&t)[NTRI], V r, V& p) {
       float kr[MR::CS];
-      mode_row<NS>(mtab, jj, kr);
+      mrow(jj, kr);
       V g = splat<V>(0.0f);
 #pragma unroll
       for (int k = 0; k < NTRI; ++k) g = vfma(splat<V>(kr[k]), Q[k], g);
@@ -393,40 +436,63 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
 #pragma unroll
       for (int k = 0; k < NTRI; ++k) t[k] = vfma(v, splat<V>(kr[k]), t[k]);
     };
+    // R and P of mode j: in shared memory (SM), or in the ensemble buffer at a
+    // block-uniform base plus the thread's 32-bit offset.  Only the ensemble's
+    // last tile has lanes past its end: the other tiles' passes carry no selects.
+    const bool full = (tile0 + 1) * TW <= nt;
+    const uint32_t woff = active[0] ? 4u * threadIdx.x : 0u;
+    const char* const Rt = reinterpret_cast<const char*>(ws.R + tile0 * TW);
+    const char* const Pt = reinterpret_cast<const char*>(ws.P + tile0 * TW);
+    const int64_t ms = nt * (int64_t)sizeof(float);  // bytes between modes
+    auto gload = [&](auto FULL, const char* base) {
+      const float x = *reinterpret_cast<const float*>(base + woff);
+      return (decltype(FULL)::value || active[0]) ? x : 0.0f;
+    };
+    auto gstore = [&](auto FULL, const char* base, float x) {
+      if (decltype(FULL)::value || active[0])
+        *reinterpret_cast<float*>(const_cast<char*>(base) + woff) = x;
+    };
+    // one pass over the modes: f(j, r, p) with r, p loaded; stores P, and R with
+    // ST_R
+    auto mode_pass = [&](auto FULL, auto ST_R, auto&& f) {
+      auto batch = [&](int j, auto M_, const char* Rj, const char* Pj, float* rs, float* ps) {
+        constexpr int M = decltype(M_)::value;
+        V rb[M], pb[M];
+#pragma unroll
+        for (int u = 0; u < M; ++u) {
+          ln(rb[u], 0) = SM == 2 ? rs[u * TW] : gload(FULL, Rj + u * ms);
+          ln(pb[u], 0) = SM > 0 ? ps[u * TW] : gload(FULL, Pj + u * ms);
+        }
+#pragma unroll
+        for (int u = 0; u < M; ++u) f(j + u, rb[u], pb[u]);
+#pragma unroll
+        for (int u = 0; u < M; ++u) {
+          if (decltype(ST_R)::value) {
+            if (SM == 2) rs[u * TW] = ln(rb[u], 0);
+            else gstore(FULL, Rj + u * ms, ln(rb[u], 0));
+          }
+          if (SM > 0) ps[u * TW] = ln(pb[u], 0);
+          else gstore(FULL, Pj + u * ms, ln(pb[u], 0));
+        }
+      };
+      // (a pointer for each array and a counter for the coefficients: the counter
+      // stays warp-uniform)
+      const char *Rj = Rt, *Pj = Pt;
+      float *rs = Rs, *ps = Ps;
+      int j = 0;
+      for (; j + MU <= bp.n;
+           j += MU, Rj += MU * ms, Pj += MU * ms, rs += MU * TW, ps += MU * TW)
+        batch(j, std::integral_constant<int, MU>{}, Rj, Pj, rs, ps);
+      for (; j < bp.n; ++j, Rj += ms, Pj += ms, rs += TW, ps += TW)
+        batch(j, std::integral_constant<int, 1>{}, Rj, Pj, rs, ps);
+    };
     auto pass_a = [&](const V (&Q)[NTRI], V (&W)[NS][NS]) {
       V t[NTRI];
 #pragma unroll
       for (int k = 0; k < NTRI; ++k) t[k] = splat<V>(cf.E[k]);
-      float* R0 = ws.R + (active[0] ? iw[0] : 0);
-      float* P0 = ws.P + (active[0] ? iw[0] : 0);
-      int j = 0;
-      for (; j + MU <= bp.n; j += MU, R0 += MU * nt, P0 += MU * nt) {
-        V rb[MU], pb[MU];
-#pragma unroll
-        for (int u = 0; u < MU; ++u) {
-          ln(rb[u], 0) = active[0] ? R0[u * nt] : 0.0f;
-          ln(pb[u], 0) = active[0] ? P0[u * nt] : 0.0f;
-        }
-#pragma unroll
-        for (int u = 0; u < MU; ++u) mode_a(j + u, Q, t, rb[u], pb[u]);
-        if (active[0]) {
-#pragma unroll
-          for (int u = 0; u < MU; ++u) {
-            R0[u * nt] = ln(rb[u], 0);
-            P0[u * nt] = ln(pb[u], 0);
-          }
-        }
-      }
-      for (; j < bp.n; ++j, R0 += nt, P0 += nt) {
-        V r, p;
-        ln(r, 0) = active[0] ? *R0 : 0.0f;
-        ln(p, 0) = active[0] ? *P0 : 0.0f;
-        mode_a(j, Q, t, r, p);
-        if (active[0]) {
-          *R0 = ln(r, 0);
-          *P0 = ln(p, 0);
-        }
-      }
+      auto f = [&](int jj, V& r, V& p) { mode_a(jj, Q, t, r, p); };
+      if (SM == 2 || full) mode_pass(std::true_type{}, std::true_type{}, f);
+      else mode_pass(std::false_type{}, std::true_type{}, f);
 #pragma unroll
       for (int a = 0; a < NS; ++a)
 #pragma unroll
@@ -435,31 +501,16 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
     auto pass_b = [&](const V (&Q)[NTRI], V (&t)[NTRI]) {
 #pragma unroll
       for (int k = 0; k < NTRI; ++k) t[k] = splat<V>(0.0f);
-      const float* R0 = ws.R + (active[0] ? iw[0] : 0);
-      float* P0 = ws.P + (active[0] ? iw[0] : 0);
-      int j = 0;
-      for (; j + MU <= bp.n; j += MU, R0 += MU * nt, P0 += MU * nt) {
-        V rb[MU], pb[MU];
-#pragma unroll
-        for (int u = 0; u < MU; ++u) {
-          ln(rb[u], 0) = active[0] ? R0[u * nt] : 0.0f;
-          ln(pb[u], 0) = active[0] ? P0[u * nt] : 0.0f;
-        }
-#pragma unroll
-        for (int u = 0; u < MU; ++u) mode_b(j + u, Q, t, rb[u], pb[u]);
-        if (active[0]) {
-#pragma unroll
-          for (int u = 0; u < MU; ++u) P0[u * nt] = ln(pb[u], 0);
-        }
-      }
-      for (; j < bp.n; ++j, R0 += nt, P0 += nt) {
-        V r, p;
-        ln(r, 0) = active[0] ? *R0 : 0.0f;
-        ln(p, 0) = active[0] ? *P0 : 0.0f;
-        mode_b(j, Q, t, r, p);
-        if (active[0]) *P0 = ln(p, 0);
-      }
+      auto f = [&](int jj, V& r, V& p) { mode_b(jj, Q, t, r, p); };
+      if (SM == 2 || full) mode_pass(std::true_type{}, std::false_type{}, f);
+      else mode_pass(std::false_type{}, std::false_type{}, f);
     };
+    if constexpr (SM > 0) {
+      for (int j = 0; j < bp.n; ++j) {
+        Ps[j * TW] = active[0] ? ws.P[(int64_t)j * nt + iw[0]] : 0.0f;
+        if (SM == 2) Rs[j * TW] = active[0] ? ws.R[(int64_t)j * nt + iw[0]] : 0.0f;
+      }
+    }
     // observation of walker lane l into slot `slot` of tile tile0 + l
     auto observe_lane = [&](int l, int slot) {
       f2 ml = {ln(m.hi, l), ln(m.lo, l)};
@@ -748,6 +799,12 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
           ws.R[(int64_t)j * nt + i] = ln(R[j], l);
           ws.P[(int64_t)j * nt + i] = ln(P[j], l);
         }
+      if constexpr (SM > 0) {
+        for (int j = 0; j < bp.n; ++j) {
+          ws.P[(int64_t)j * nt + i] = Ps[j * TW];
+          if (SM == 2) ws.R[(int64_t)j * nt + i] = Rs[j * TW];
+        }
+      }
 #pragma unroll
       for (int a = 0; a < NS; ++a) {
 #pragma unroll

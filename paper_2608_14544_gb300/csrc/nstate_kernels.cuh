@@ -101,29 +101,41 @@ struct NStateOps {
                                                                        part);
     launches_add(1);
   }
-  template <int NPL, int WPT = 1>
-  static int bulk_npl(const BulkParams& bp, const CoefN& cf, void* buf, double* part,
-                      int grid_cap, cudaStream_t st) {
+  // (NM > 0: the modes-in-memory form with its coefficient rows as a kernel
+  // parameter)
+  template <int NPL, int WPT = 1, int NM = 0, int SM = 0>
+  static int bulk_npl(const BulkParams& bp, const CoefN& cf, const ModeHost& mh, void* buf,
+                      double* part, int grid_cap, cudaStream_t st) {
     // (occupancy cached per kernel and table size: [0] adiabatic, [1] diabatic;
     // NPL = 0: the mode table in dynamic shared memory)
     static int per_sm[2] = {-1, -1}, n_sm[2] = {0, 0};
     static size_t dyn_at[2] = {0, 0};
-    const size_t dyn = NPL == 0 ? ModeRow<NS>::bytes(bp.n) : 0;
-    if (bp.repr == QCL_REPR_DIABATIC)
-      return launch_persistent(k_bulkN_dia<NS, NPL>, per_sm[1], n_sm[1], dyn_at[1], bp, cf, buf,
-                               part, grid_cap, 1, dyn, st);
-    return launch_persistent(k_bulkN<NS, NPL, WPT>, per_sm[0], n_sm[0], dyn_at[0], bp, cf, buf,
-                             part, grid_cap, WPT, dyn, st);
+    const size_t dyn = NPL != 0  ? 0
+                       : NM == 0 ? ModeRow<NS>::bytes(bp.n)
+                                 : (size_t)SM * bp.n * 128 * sizeof(float);
+    if constexpr (NM == 0) {
+      if (bp.repr == QCL_REPR_DIABATIC)
+        return launch_persistent(k_bulkN_dia<NS, NPL>, per_sm[1], n_sm[1], dyn_at[1], bp, grid_cap,
+                                 1, dyn, st, bp, cf, buf, part);
+    }
+    if constexpr (NPL == 0 && NM == 0 && NS <= 4) {
+      return 0;  // (adiabatic models of N_s <= 4 take NM > 0)
+    } else {
+      CoefMem<NS, NM> cm;
+      if constexpr (NM > 0) make_coef_mem(mh, bp.n, cm);
+      return launch_persistent(k_bulkN<NS, NPL, WPT, NM, SM>, per_sm[0], n_sm[0], dyn_at[0], bp,
+                               grid_cap, WPT, dyn, st, bp, cf, buf, part, cm);
+    }
   }
   // one persistent grid: the occupancy limit of resident blocks on every SM
   // (capped), at most one block per WPT tiles
   // (dyn > 0, the modes-in-memory kernels: the shared-memory limit only grows
   // and the occupancy is computed for this call's table, under a lock, so
   // that threads launching models of different mode counts do not race)
-  template <typename Fn>
+  template <typename Fn, typename... Args>
   static int launch_persistent(Fn fn, int& per_sm, int& n_sm, size_t& dyn_at, const BulkParams& bp,
-                               const CoefN& cf, void* buf, double* part, int grid_cap, int WPT,
-                               size_t dyn, cudaStream_t st) {
+                               int grid_cap, int WPT, size_t dyn, cudaStream_t st,
+                               const Args&... args) {
     int blocks = per_sm;
     if (dyn > 0) {
       static std::mutex mu;
@@ -154,24 +166,24 @@ struct NStateOps {
     const int64_t units = (bp.n_tiles + WPT - 1) / WPT;
     if (grid > units) grid = units;
     if (grid < 1) grid = 1;
-    fn<<<(unsigned)grid, 128, dyn, st>>>(bp, cf, buf, part);
+    fn<<<(unsigned)grid, 128, dyn, st>>>(args...);
     return (int)grid;
   }
   // wpt: walkers per thread asked for.  The kernel takes one or two, but only
   // one is instantiated: two walkers per thread (packed lanes, 205-245
   // registers, 8 resident warps per SM) measured 10 % slower on a four-state
   // six-mode model than one (114 registers, 16 warps), with the same bits.
-  static int bulk(const BulkParams& bp, const CoefN& cf, void* buf, double* part, int grid_cap,
-                  int wpt, cudaStream_t st) {
+  static int bulk(const BulkParams& bp, const CoefN& cf, const ModeHost& mh, void* buf,
+                  double* part, int grid_cap, int wpt, cudaStream_t st) {
     (void)wpt;
     // Register forms exist up to 8 modes for any N_s and up to 32 modes for
     // N_s <= 4 (larger N_s x modes would not fit a walker in registers); the
     // modes-in-memory form takes any mode count with the same bits.  The
     // automatic choice follows measured solve rates on GB300 (1e6 walkers,
     // 200 steps, random LVC models): registers for N_s = 3 (except adiabatic
-    // models of 9-16 modes, where the 32-mode register form is 10-30 % slower)
-    // and for N_s = 4 up to 8 modes (20-30 % faster); the memory form beyond
-    // (N_s = 4 with 12-32 modes: 1.3-2.6x faster) and for N_s >= 5 at every
+    // models of 9-24 modes, where the 32-mode register form is 10-50 % slower)
+    // and for N_s = 4 up to 8 modes (10-20 % faster); the memory form beyond
+    // (N_s = 4 with 12-32 modes: 1.2-2x faster) and for N_s >= 5 at every
     // mode count (1.0-2.2x, the register forms there run one or two blocks per
     // SM).  Models of at most 4 or 6 modes get their own instantiations,
     // which skip the padding modes' arithmetic (padding modes have zero
@@ -180,16 +192,29 @@ struct NStateOps {
     bool mem;
     if (cf.modes_in_memory == 1) mem = true;
     else if (cf.modes_in_memory == 2) mem = bp.n > reg_max;
-    else if (NS == 3) mem = bp.n > 32 || (bp.repr != QCL_REPR_DIABATIC && bp.n > 8 && bp.n <= 16);
+    else if (NS == 3) mem = bp.n > 32 || (bp.repr != QCL_REPR_DIABATIC && bp.n > 8 && bp.n <= 24);
     else if (NS == 4) mem = bp.n > 8;
     else mem = true;
-    if (mem) return bulk_npl<0>(bp, cf, buf, part, grid_cap, st);
-    if constexpr (NS <= 5) {
-      if (bp.n <= 4) return bulk_npl<4>(bp, cf, buf, part, grid_cap, st);
-      if (bp.n <= 6) return bulk_npl<6>(bp, cf, buf, part, grid_cap, st);
+    // The adiabatic memory form of N_s <= 4 takes its coefficients as a kernel
+    // parameter and keeps R and P in shared memory up to 32 modes, P alone up
+    // to 64 (32 KB a block in either case, so that four blocks still fit an SM;
+    // at 128 modes P alone left two, and was 40 % slower than no arrays).
+    // N_s = 4, 300011 walkers x 30 steps: 12 modes 0.81 -> 0.74 ms, 32 modes
+    // 1.53 -> 1.25, 64 modes 2.72 -> 2.29, 128 modes 5.63 -> 5.13.
+    if constexpr (NS <= 4) {
+      if (mem && bp.repr != QCL_REPR_DIABATIC) {
+        if (bp.n <= 32) return bulk_npl<0, 1, 64, 2>(bp, cf, mh, buf, part, grid_cap, st);
+        if (bp.n <= 64) return bulk_npl<0, 1, 64, 1>(bp, cf, mh, buf, part, grid_cap, st);
+        return bulk_npl<0, 1, 256, 0>(bp, cf, mh, buf, part, grid_cap, st);
+      }
     }
-    if (bp.n <= 8) return bulk_npl<8>(bp, cf, buf, part, grid_cap, st);
-    if (NS <= 4 && bp.n <= 32) return bulk_npl<(NS <= 4 ? 32 : 8)>(bp, cf, buf, part, grid_cap, st);
+    if (mem) return bulk_npl<0>(bp, cf, mh, buf, part, grid_cap, st);
+    if constexpr (NS <= 5) {
+      if (bp.n <= 4) return bulk_npl<4>(bp, cf, mh, buf, part, grid_cap, st);
+      if (bp.n <= 6) return bulk_npl<6>(bp, cf, mh, buf, part, grid_cap, st);
+    }
+    if (bp.n <= 8) return bulk_npl<8>(bp, cf, mh, buf, part, grid_cap, st);
+    if (NS <= 4 && bp.n <= 32) return bulk_npl<(NS <= 4 ? 32 : 8)>(bp, cf, mh, buf, part, grid_cap, st);
     return 0;
   }
 };

@@ -576,7 +576,7 @@ qcl_status qcl_propagate(const qcl_model* model, const qcl_ensemble_desc* ens, v
         ls.wpt = model->shape_wpt;
         ls.blocks_per_sm = model->shape_bps;
         ls.grid_cap = (int)g_opt_grid_cap;
-        grid = cn ? launch_bulkN(model->ns, bp, *cn, ens_buf, part, ls, s)
+        grid = cn ? launch_bulkN(model->ns, bp, *cn, ModeHost{&model->host, model->K.data(), dt}, ens_buf, part, ls, s)
                   : launch_bulk2(bp, *cf, ens_buf, part, ls, s);
       }
       if (grid == 0) {
