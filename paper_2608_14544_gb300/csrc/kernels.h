@@ -241,6 +241,7 @@ struct SpawnHeader {
   int64_t n_live[2];  // live walkers of set 0 and set 1
   int32_t drop;       // set by the scan when a step's children do not fit
   int32_t pad;
+  unsigned long long total[3];  // the chained steps' child counts (step mod 3)
 };
 constexpr size_t kSpawnHeaderOff = 64;  // after EnsHeader, inside the first 256 bytes
 
@@ -323,7 +324,7 @@ void launch_spawn_observe(const DevModel* dm, const void* buf, int64_t capacity,
                           int set, double* part, cudaStream_t st);
 // Grid of the spawning kernels: a few blocks per SM, each walking groups of 256
 // walkers up to the live count (which the host does not know).
-unsigned spawn_grid(int64_t capacity);
+unsigned spawn_grid(int64_t capacity, int per_sm = 8);
 // The block-count scan and the family starts, for either precision's layout.
 void launch_spawn_scan(void* buf, int64_t capacity, int n, int64_t n0, int precision, int ns, int64_t step0,
                        int64_t step, cudaStream_t st);
@@ -347,12 +348,12 @@ int launch_spawnN_step32(int ns, const BulkParams& bp, const CoefN& cf, void* bu
 void launch_spawnN_observe32(int ns, const BulkParams& bp, const CoefN& cf, const void* buf,
                              int64_t capacity, int64_t n0, int set, double* part,
                              cudaStream_t st);
-// FP32-bulk spawning (two states, n <= 32 modes): sample, one step (step
-// kernel, scan, scatter), family observation.
+// FP32-bulk spawning (two states): sample, steps [step, step + len) of a call that
+// began at step0, family observation.
 void launch_spawn_sample32(const DevModel& host, const SampleParams& sp, int64_t capacity, void* buf,
                            cudaStream_t st);
-int launch_spawn_step32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t capacity,
-                        int64_t n0, int64_t step0, int64_t step, cudaStream_t st);
+void launch_spawn_steps32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t capacity,
+                          int64_t n0, int64_t step0, int64_t step, int64_t len, cudaStream_t st);
 void launch_spawn_observe32(const BulkParams& bp, const Coef2& cf, const void* buf, int64_t capacity,
                             int64_t n0, int set, double* part, cudaStream_t st);
 

@@ -999,19 +999,23 @@ qcl_status qcl_spawn_propagate(const qcl_model* model, const qcl_ensemble_desc* 
     launch_fold(part, row, fold, OL.n_tiles, q2, 1, s);
   };
   if (step0 == 0) observe(rows, 0);
-  for (int64_t t = step0; t < step0 + n_steps; ++t) {
+  const int64_t end = step0 + n_steps;
+  for (int64_t t = step0; t < end;) {
+    // (two states in FP32: the steps up to the next output time at once)
+    const int64_t len = f32 && !f32n ? std::min<int64_t>(end, (t / out_stride + 1) * out_stride) - t : 1;
     {
       TimedLaunch tl(1, s);
       if (f32n)
         launch_spawnN_step32(model->ns, bp, *cn, buf, capacity, n0, step0, t, s);
       else if (f32)
-        launch_spawn_step32(bp, *cf, buf, capacity, n0, step0, t, s);
+        launch_spawn_steps32(bp, *cf, buf, capacity, n0, step0, t, len, s);
       else if (model->ns > 2)
         launch_spawnN_step(model->dev, model->ns, buf, capacity, model->n, n0, step0, t, dt, ens->seed, s);
       else
         launch_spawn_step(model->host, buf, capacity, n0, step0, t, dt, ens->seed, s);
     }
-    if ((t + 1) % out_stride == 0) observe(rows + (size_t)((t + 1) / out_stride) * q2, t + 1);
+    t += len;
+    if (t % out_stride == 0) observe(rows + (size_t)(t / out_stride) * q2, t);
   }
   delete cf;
   delete cn;

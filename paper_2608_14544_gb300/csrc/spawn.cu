@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(256) k_spawn_observe(const DevModel* __restric
 
 }  // namespace
 
-unsigned spawn_grid(int64_t capacity) {
+unsigned spawn_grid(int64_t capacity, int per_sm) {
   static int n_sm = 0;
   if (n_sm == 0) {
     int dev = 0;
@@ -320,7 +320,7 @@ unsigned spawn_grid(int64_t capacity) {
     if (n_sm < 1) n_sm = 1;
   }
   const int64_t groups = (capacity + 255) / 256;
-  const int64_t g = (int64_t)8 * n_sm;
+  const int64_t g = (int64_t)per_sm * n_sm;
   return (unsigned)(groups < g ? (groups > 0 ? groups : 1) : g);
 }
 

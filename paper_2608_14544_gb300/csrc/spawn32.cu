@@ -1,10 +1,9 @@
 // spawn32.cu -- trajectory spawning in FP32 bulk precision (two states, any
 // mode count, either representation).  The same scheme and walker order as the
-// FP64 spawning kernels (spawn.cu): one step per launch, a child inserted right
-// after its parent by the deterministic count / scan / scatter; the walker's
-// arithmetic is that of the FP32-bulk kernels (compensated phase and weight
-// pairs with a carried exponent), with the state read from and written to HBM
-// every step.  Family observation in FP64 from the walkers' FP32 contributions.
+// FP64 spawning kernels (spawn.cu), a child inserted right after its parent; the
+// walker's arithmetic is that of the FP32-bulk kernels (compensated phase and
+// weight pairs with a carried exponent), with the state read from and written to
+// memory every step.  Family observation in FP64 from the walkers' FP32 contributions.
 #include "bulk2.cuh"
 #include "model.h"
 #include "reduce.cuh"
@@ -27,7 +26,7 @@ struct Set32 {
 };
 
 __device__ __forceinline__ Set32 set32(void* buf, const SpawnLayout& L, int set) {
-  char* b = (char*)buf + L.set_off[set];
+  char* b = (char*)buf + (set ? L.set_off[1] : L.set_off[0]);
   return {(float*)(b + L.R),     (float*)(b + L.P),    (float*)(b + L.m),
           (float*)(b + L.mlo),   (int32_t*)(b + L.mexp), (float*)(b + L.phi),
           (float*)(b + L.philo), (uint16_t*)(b + L.ab), (uint64_t*)(b + L.id),
@@ -82,19 +81,327 @@ __global__ void __launch_bounds__(256) k_spawn_sample32(const Sample32 sp, int64
   w.fam[i] = (uint32_t)i;
 }
 
-// One step of every live walker of set `src` (in place); children to the
-// per-parent staging, each block's child count to bsum.
-// NPL = 0: the modes stay in memory (any mode count), read and written back
-// mode by mode with the register form's operations in its order (the same
-// bits): one pass for the diabatic step, three for the adiabatic one (a(R_n),
-// b(R_n); first half kick, drift, a and b at R_{n+1}; second half kick and the
-// coupling sums).
+__device__ __forceinline__ uint16_t pair_word(const Scal& z) {
+  return (uint16_t)((z.sa > 0.0f ? 1 : 0) | ((z.q & 3) << 4) | ((z.sb > 0.0f ? 1 : 0) << 8));
+}
+
+// The phase pair is renormalised, and wrapped past 2^10 rad, at the end of
+// every Philox block (absolute steps 4k + 3).
+__device__ __forceinline__ void spawn_phase_end(Scal& z, int64_t step) {
+  if ((step & 3) == 3) {
+    z.ph = two_sum(z.ph.hi, z.ph.lo);
+    phase_wrap(z);
+  }
+}
+
+// What a step reports: a non-finite child or phase, a degenerate gap.
+__device__ __forceinline__ void spawn_report(EnsHeader* hdr, const Scal& z, bool hop,
+                                             const Scal& child, unsigned int deg) {
+  const unsigned bad = (hop && !isfinite(child.m.hi) ? 1u : 0u) + (!isfinite(z.ph.hi) ? 1u : 0u);
+  if (bad) {
+    atomicAdd(&hdr->n_nonfinite, (unsigned long long)bad);
+    atomicOr(&hdr->flags, QCL_FLAG_NONFINITE);
+  }
+  if (deg) {
+    atomicAdd(&hdr->n_degenerate, 1ull);
+    atomicOr(&hdr->flags, QCL_FLAG_DEGENERATE);
+  }
+}
+
+// A walker of the chained steps, modes in registers.
+template <int NPL>
+struct SWalker {
+  Walker<NPL> w;
+  f2 m, ph;
+  int32_t me;
+  uint16_t ab;
+};
+
+template <int NPL>
+__device__ __forceinline__ void put_walker(const Set32& s, int64_t cap, int n, int64_t pos,
+                                           const SWalker<NPL>& x, uint64_t id, uint32_t fam) {
+#pragma unroll
+  for (int j = 0; j < NPL; ++j)
+    if (j < n) {
+      s.R[(int64_t)j * cap + pos] = x.w.R[j];
+      s.P[(int64_t)j * cap + pos] = x.w.P[j];
+    }
+  s.mh[pos] = x.m.hi;
+  s.ml[pos] = x.m.lo;
+  s.me[pos] = x.me;
+  s.ph[pos] = x.ph.hi;
+  s.pl[pos] = x.ph.lo;
+  s.ab[pos] = x.ab;
+  s.id[pos] = id;
+  s.fam[pos] = fam;
+}
+
+// One step of the walker x (random stream id) in registers: x moves to the next
+// step (its weight and pair stay), and where its test fires the result is true
+// and cm, cme, cab are the child's weight and pair.  REPORT counts degenerate
+// gaps and non-finite values in the header.
 template <int NPL, int KIND, bool DIA>
+__device__ __forceinline__ bool step_walker(const BulkParams& bp, const CoefLocal<NPL>& cf,
+                                            EnsHeader* hdr, int64_t step, SWalker<NPL>& x,
+                                            uint64_t id, f2& cm, int32_t& cme, uint16_t& cab,
+                                            bool report) {
+  using CF = CoefLocal<NPL>;
+  Walker<NPL>& w = x.w;
+  Scal z;
+  z.m = x.m;
+  z.mexp = x.me;
+  z.ph = x.ph;
+  z.sa = sgn(x.ab & 0xf);
+  z.sb = sgn((x.ab >> 8) & 0xf);
+  z.q = DIA ? (int)((x.ab >> 4) & 3u) : 0;
+  z.A = bp.a0;
+  z.B = bp.b0;
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) {
+    z.A = __fmaf_rn(cf.a[j], w.R[j], z.A);
+    if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
+  }
+  closed_form(z);
+  const u4 wd = philox_draw(bp.seed, (uint32_t)(step >> 2), id, kPurposeHop);
+  const uint32_t word = word_of(wd, (int)(step & 3));
+  unsigned int deg = 0;
+  Scal child;
+  bool hop;
+  const float hsab = bp.hdt * 0.5f * (z.sa + z.sb);
+  if (DIA) {
+    kick_dia<NPL, KIND, CF>(w, cf, hsab);
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) w.R[j] = __fmaf_rn(cf.dtm[j], w.P[j], w.R[j]);
+    const float a_old = z.A;
+    z.A = bp.a0;
+    if (KIND == 1) z.B = bp.b0;
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) {
+      z.A = __fmaf_rn(cf.a[j], w.R[j], z.A);
+      if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
+    }
+    kick_dia<NPL, KIND, CF>(w, cf, hsab);
+    hop = spawn_transition<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, child);
+  } else {
+    kick<NPL, KIND, CF>(w, cf, hsab * z.c2, hsab * z.s2);
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) w.R[j] = __fmaf_rn(cf.dtm[j], w.P[j], w.R[j]);
+    const float r_old = z.r;
+    z.A = bp.a0;
+    z.B = bp.b0;
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) {
+      z.A = __fmaf_rn(cf.a[j], w.R[j], z.A);
+      if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
+    }
+    closed_form(z);
+    kick<NPL, KIND, CF>(w, cf, hsab * z.c2, hsab * z.s2);
+    float Av = 0.0f, Bv = 0.0f;
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) {
+      Av = __fmaf_rn(cf.am[j], w.P[j], Av);
+      if (KIND == 1) Bv = __fmaf_rn(cf.bm[j], w.P[j], Bv);
+    }
+    hop = spawn_transition<KIND, false>(z, r_old, Av, Bv, word, bp, deg, child);
+  }
+  spawn_phase_end(z, step);
+  x.ph = z.ph;
+  if (hop) {
+    renorm(child.m, child.mexp);
+    cm = child.m;
+    cme = child.mexp;
+    cab = pair_word(child);
+  }
+  if (report) spawn_report(hdr, z, hop, child, deg);
+  return hop;
+}
+
+// The chained steps' counts: children of each 256-walker group of the current
+// set at step s in array s mod 3 (the space of bsum and boff), their sum in
+// total[s mod 3].
+__device__ __forceinline__ unsigned int* chain_counts(void* buf, const SpawnLayout& L, int k) {
+  char* b = (char*)buf;
+  return (unsigned int*)(k == 0 ? b + L.bsum : (k == 1 ? b + L.boff : b + L.boff + 4 * L.n_blocks));
+}
+
+// Adds this warp's firing walkers (bal, lane l at position pos0 + rank) to the
+// counts of the groups their positions fall in.
+__device__ __forceinline__ void add_counts(unsigned int* cnt, bool fires, int64_t pos) {
+  const int lane = threadIdx.x & 31;
+  const unsigned act = __ballot_sync(0xffffffffu, fires);
+  if (!act) return;
+  // positions ascend over the lanes and span at most two groups
+  const int64_t g = pos >> 8;
+  const int64_t g_lo = __shfl_sync(0xffffffffu, g, __ffs(act) - 1);
+  const unsigned lo = __ballot_sync(0xffffffffu, fires && g == g_lo);
+  if (lane == __ffs(act) - 1) atomicAdd(cnt + g_lo, (unsigned)__popc(lo));
+  const unsigned up = act & ~lo;
+  if (up && lane == __ffs(up) - 1) atomicAdd(cnt + g, (unsigned)__popc(up));
+}
+
+// One spawning step of the whole ensemble in one pass: set s & 1 to the other.
+// The children of this step are known before it starts: the launch before has
+// evaluated, beside its own step, which of its walkers fire at the next one, and
+// counted them by the group of 256 positions they stand in.  So a block learns
+// the children before its walkers by adding the counts of the groups before
+// them, steps its walkers in registers, writes each with its child straight to
+// its place, and evaluates the step after for the counts of the next launch
+// (FIRST only counts, for a call's first step).  Nothing waits inside a launch,
+// and an overflow is known at its start: then the step's children are dropped.
+//
+// What bounds it: instruction issue at 1e6 walkers (698 instructions a warp of
+// walkers, of which the two evaluations of the step are 360; 40 us a step against
+// 15 us for its bytes), launch latency below some 1e5 (8-12 us a step).  1e5
+// initial one-mode walkers growing to 1.55e6 over 400 steps: 10.0 ms of device
+// time, where a step in place, a one-block scan and a scatter took 15.9 ms.  One
+// cooperative launch for many steps, with a decoupled look-back over the groups'
+// counts and a grid barrier, was slower (13.6 ms): a poll of another die's word
+// costs about a microsecond, and a step needs several in a row.
+template <int NPL, int KIND, bool DIA, bool FIRST>
+__global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
+    k_spawn_chain32(const BulkParams bp, const CoefLocal<NPL> cf, const SpawnLayout L, void* buf,
+                    int64_t cap, int64_t step) {
+  __shared__ int wcnt[2][8];
+  __shared__ unsigned long long wsum[8];
+  EnsHeader* hdr = (EnsHeader*)buf;
+  SpawnHeader* sh = hdr_spawn(buf);
+  // (FIRST counts the step itself; otherwise the step after it)
+  const int src = (int)(step & 1), k3 = (int)(step % 3);
+  const int64_t n_live = sh->n_live[src];
+  const int64_t total = FIRST ? 0 : (int64_t)sh->total[k3];
+  if (hdr->step != bp.step0) {  // uniform over the grid
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&hdr->flags, QCL_FLAG_STEP_MISMATCH);
+    return;
+  }
+  const int kn = FIRST ? k3 : (k3 + 1) % 3, kz = (k3 + 2) % 3;
+  unsigned int* const cnt = chain_counts(buf, L, k3);
+  unsigned int* const nxt = chain_counts(buf, L, kn);
+  unsigned int* const clr = chain_counts(buf, L, kz);
+  const bool drop = n_live + total > cap;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // a contiguous run of groups for each block
+  const int64_t groups = (n_live + 255) / 256;
+  const int64_t per = (groups + gridDim.x - 1) / gridDim.x;
+  const int64_t g0 = min((int64_t)blockIdx.x * per, groups), g1 = min(g0 + per, groups);
+  const Set32 s = set32(buf, L, src), d = set32(buf, L, src ^ 1);
+  SWalker<NPL> x;
+  uint64_t id = 0;
+  uint32_t fam = 0;
+  auto load = [&](int64_t g) {
+    const int64_t i = g * 256 + threadIdx.x;
+    const int64_t ii = i < n_live ? i : 0;
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) {
+      const bool on = j < bp.n;
+      x.w.R[j] = on ? s.R[(int64_t)j * cap + ii] : 0.0f;
+      x.w.P[j] = on ? s.P[(int64_t)j * cap + ii] : 0.0f;
+    }
+    x.m = {s.mh[ii], s.ml[ii]};
+    x.me = s.me[ii];
+    x.ph = {s.ph[ii], s.pl[ii]};
+    x.ab = s.ab[ii];
+    id = s.id[ii];
+    fam = s.fam[ii];
+  };
+  if (g0 < g1) load(g0);  // (in flight while the prefix is added up)
+  int64_t prefix = 0;
+  if (!FIRST) {
+    for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < L.n_blocks;
+         k += (int64_t)gridDim.x * 256)
+      clr[k] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      sh->total[kz] = 0;
+      sh->n_live[src ^ 1] = drop ? n_live : n_live + total;
+      if (drop) atomicOr(&hdr->flags, QCL_FLAG_SPAWN_OVERFLOW);
+    }
+    if (!drop && g0 < g1) {
+      unsigned long long sum = 0;
+      for (int64_t k = threadIdx.x; k < g0; k += 256) sum += cnt[k];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+      if (lane == 0) wsum[warp] = sum;
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < 8; ++k) prefix += (int64_t)wsum[k];
+    }
+  }
+  unsigned int found = 0;  // firing walkers this thread's warp counted (lane 0)
+  for (int64_t g = g0; g < g1; ++g) {
+    const int64_t i = g * 256 + threadIdx.x;
+    const bool live = i < n_live;
+    if (g > g0) load(g);
+    // phase 0: the step itself; 1: the walkers' next step; 2: their children's.
+    // One copy of the step's code, so that a walker's test comes out the same
+    // when it is counted and when it is taken.
+    SWalker<NPL> xc;      // the children
+    uint64_t idc = 0;
+    bool hop = false;
+    int64_t pos = i;
+#pragma unroll 1
+    for (int phase = FIRST ? 1 : 0; phase < 3; ++phase) {
+      if (phase == 2) {
+        if (FIRST || !__any_sync(0xffffffffu, hop)) break;
+        x = xc;
+        id = idc;
+      }
+      f2 cm;
+      int32_t cme;
+      uint16_t cab;
+      const bool fires = step_walker<NPL, KIND, DIA>(bp, cf, hdr, FIRST || phase == 0 ? step : step + 1,
+                                                     x, id, cm, cme, cab, phase == 0 && live);
+      if (phase == 0) {
+        hop = fires && live && !drop;
+        const unsigned bal = __ballot_sync(0xffffffffu, hop);
+        int* const wc = wcnt[(g - g0) & 1];  // (two in turn: one barrier a group)
+        if (lane == 0) wc[warp] = __popc(bal);
+        __syncthreads();
+        int before = __popc(bal & ((1u << lane) - 1u)), c = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          before += k < warp ? wc[k] : 0;
+          c += wc[k];
+        }
+        pos = i + prefix + before;
+        prefix += c;
+        if (live) put_walker(d, cap, bp.n, pos, x, id, fam);
+        if (hop) {
+          xc = x;
+          xc.m = cm;
+          xc.me = cme;
+          xc.ab = cab;
+          idc = child_id32(bp.seed, step, id);
+          put_walker(d, cap, bp.n, pos + 1, xc, idc, fam);
+        }
+      } else {
+        const bool f = fires && (phase == 1 ? live : hop);
+        add_counts(nxt, f, phase == 1 ? pos : pos + 1);
+        found += __popc(__ballot_sync(0xffffffffu, f));
+      }
+    }
+  }
+  if (lane == 0 && found) atomicAdd(&sh->total[kn], (unsigned long long)found);
+}
+
+// The counts and totals of a call's first step start at zero.
+__global__ void __launch_bounds__(256) k_spawn_chain_clear(void* buf, int64_t cap, int n,
+                                                           int64_t n0) {
+  const SpawnLayout L = SpawnLayout::make(cap, n, n0, QCL_PREC_FP32_BULK);
+  for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < L.n_blocks;
+       k += (int64_t)gridDim.x * 256)
+    for (int a = 0; a < 3; ++a) chain_counts(buf, L, a)[k] = 0u;
+  if (blockIdx.x == 0 && threadIdx.x < 3) hdr_spawn(buf)->total[threadIdx.x] = 0;
+}
+
+// Any mode count, the modes in memory: one step of every live walker of set
+// `src` (in place); children to the per-parent staging, each block's child count
+// to bsum.  R and P are read and written back mode by mode with the
+// register form's operations in its order (the same bits): one pass for the diabatic
+// step, three for the adiabatic one (a(R_n), b(R_n); first half kick, drift, a
+// and b at R_{n+1}; second half kick and the coupling sums).
+template <int KIND, bool DIA>
 __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const Coef2 cf,
                                                       void* buf, int64_t cap, int64_t n0,
                                                       int64_t step) {
-  constexpr bool MEM = NPL == 0;
-  constexpr int NR = MEM ? 1 : NPL;
   const SpawnLayout L = SpawnLayout::make(cap, bp.n, n0, QCL_PREC_FP32_BULK);
   EnsHeader* hdr = (EnsHeader*)buf;
   const int src = (int)(step & 1);
@@ -111,13 +418,6 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
     int flag = 0;
     if (i < n_live) {
       const Set32 s = set32(buf, L, src);
-      Walker<NR> w;
-  #pragma unroll
-      for (int j = 0; j < NPL; ++j) {
-        const bool on = j < bp.n;
-        w.R[j] = on ? s.R[(int64_t)j * cap + i] : 0.0f;
-        w.P[j] = on ? s.P[(int64_t)j * cap + i] : 0.0f;
-      }
       Scal z;
       z.m = {s.mh[i], s.ml[i]};
       z.mexp = s.me[i];
@@ -128,17 +428,10 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
       z.q = DIA ? (int)((ab >> 4) & 3u) : 0;
       z.A = bp.a0;
       z.B = bp.b0;
-      if constexpr (MEM) {
-        for (int j = 0; j < bp.n; ++j) {
-          const float r = s.R[(int64_t)j * cap + i];
-          z.A = __fmaf_rn(cf.a[j], r, z.A);
-          if (KIND == 1) z.B = __fmaf_rn(cf.b[j], r, z.B);
-        }
-      }
-  #pragma unroll
-      for (int j = 0; j < NPL; ++j) {
-        z.A = __fmaf_rn(cf.a[j], w.R[j], z.A);
-        if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
+      for (int j = 0; j < bp.n; ++j) {
+        const float r = s.R[(int64_t)j * cap + i];
+        z.A = __fmaf_rn(cf.a[j], r, z.A);
+        if (KIND == 1) z.B = __fmaf_rn(cf.b[j], r, z.B);
       }
       closed_form(z);
       const u4 wd = philox_draw(bp.seed, (uint32_t)(step >> 2), s.id[i], kPurposeHop);
@@ -147,104 +440,56 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
       Scal child;
       bool hop;
       const float hsab = bp.hdt * 0.5f * (z.sa + z.sb);
-      if constexpr (MEM) {
-        // P += dt/2 F with the pair's force (kick / kick_dia of one mode)
-        auto kick1 = [&](int j, float r, float p, float hu, float hv) {
-          p = __fmaf_rn(-cf.hk[j], r, p);
-          if (KIND == 1) p = __fadd_rn(p, -cf.hs[j]);
-          if (DIA) return __fmaf_rn(hsab, cf.a[j], p);
-          p = __fmaf_rn(hu, -cf.a[j], p);
-          if (KIND == 1) p = __fmaf_rn(hv, -cf.b[j], p);
-          return p;
-        };
-        if (DIA) {
-          const float a_old = z.A;
-          z.A = bp.a0;
-          if (KIND == 1) z.B = bp.b0;
-          for (int j = 0; j < bp.n; ++j) {
-            float r = s.R[(int64_t)j * cap + i], p = s.P[(int64_t)j * cap + i];
-            p = kick1(j, r, p, 0.0f, 0.0f);
-            r = __fmaf_rn(cf.dtm[j], p, r);
-            z.A = __fmaf_rn(cf.a[j], r, z.A);
-            if (KIND == 1) z.B = __fmaf_rn(cf.b[j], r, z.B);
-            s.R[(int64_t)j * cap + i] = r;
-            s.P[(int64_t)j * cap + i] = kick1(j, r, p, 0.0f, 0.0f);
-          }
-          hop = spawn_transition<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, child);
-        } else {
-          const float hu = hsab * z.c2, hv = hsab * z.s2;
-          const float r_old = z.r;
-          z.A = bp.a0;
-          z.B = bp.b0;
-          for (int j = 0; j < bp.n; ++j) {
-            float r = s.R[(int64_t)j * cap + i], p = s.P[(int64_t)j * cap + i];
-            p = kick1(j, r, p, hu, hv);
-            r = __fmaf_rn(cf.dtm[j], p, r);
-            z.A = __fmaf_rn(cf.a[j], r, z.A);
-            if (KIND == 1) z.B = __fmaf_rn(cf.b[j], r, z.B);
-            s.R[(int64_t)j * cap + i] = r;
-            s.P[(int64_t)j * cap + i] = p;
-          }
-          closed_form(z);
-          const float hu2 = hsab * z.c2, hv2 = hsab * z.s2;
-          float Av = 0.0f, Bv = 0.0f;
-          for (int j = 0; j < bp.n; ++j) {
-            const float r = s.R[(int64_t)j * cap + i];
-            const float p = kick1(j, r, s.P[(int64_t)j * cap + i], hu2, hv2);
-            Av = __fmaf_rn(cf.am[j], p, Av);
-            if (KIND == 1) Bv = __fmaf_rn(cf.bm[j], p, Bv);
-            s.P[(int64_t)j * cap + i] = p;
-          }
-          hop = spawn_transition<KIND, false>(z, r_old, Av, Bv, word, bp, deg, child);
-        }
-      } else if (DIA) {
-        kick_dia<NPL, KIND, Coef2>(w, cf, hsab);
-  #pragma unroll
-        for (int j = 0; j < NPL; ++j) w.R[j] = __fmaf_rn(cf.dtm[j], w.P[j], w.R[j]);
+      // P += dt/2 F with the pair's force (kick / kick_dia of one mode)
+      auto kick1 = [&](int j, float r, float p, float hu, float hv) {
+        p = __fmaf_rn(-cf.hk[j], r, p);
+        if (KIND == 1) p = __fadd_rn(p, -cf.hs[j]);
+        if (DIA) return __fmaf_rn(hsab, cf.a[j], p);
+        p = __fmaf_rn(hu, -cf.a[j], p);
+        if (KIND == 1) p = __fmaf_rn(hv, -cf.b[j], p);
+        return p;
+      };
+      if (DIA) {
         const float a_old = z.A;
         z.A = bp.a0;
         if (KIND == 1) z.B = bp.b0;
-  #pragma unroll
-        for (int j = 0; j < NPL; ++j) {
-          z.A = __fmaf_rn(cf.a[j], w.R[j], z.A);
-          if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
+        for (int j = 0; j < bp.n; ++j) {
+          float r = s.R[(int64_t)j * cap + i], p = s.P[(int64_t)j * cap + i];
+          p = kick1(j, r, p, 0.0f, 0.0f);
+          r = __fmaf_rn(cf.dtm[j], p, r);
+          z.A = __fmaf_rn(cf.a[j], r, z.A);
+          if (KIND == 1) z.B = __fmaf_rn(cf.b[j], r, z.B);
+          s.R[(int64_t)j * cap + i] = r;
+          s.P[(int64_t)j * cap + i] = kick1(j, r, p, 0.0f, 0.0f);
         }
-        kick_dia<NPL, KIND, Coef2>(w, cf, hsab);
         hop = spawn_transition<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, child);
       } else {
-        kick<NPL, KIND, Coef2>(w, cf, hsab * z.c2, hsab * z.s2);
-  #pragma unroll
-        for (int j = 0; j < NPL; ++j) w.R[j] = __fmaf_rn(cf.dtm[j], w.P[j], w.R[j]);
+        const float hu = hsab * z.c2, hv = hsab * z.s2;
         const float r_old = z.r;
         z.A = bp.a0;
         z.B = bp.b0;
-  #pragma unroll
-        for (int j = 0; j < NPL; ++j) {
-          z.A = __fmaf_rn(cf.a[j], w.R[j], z.A);
-          if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
+        for (int j = 0; j < bp.n; ++j) {
+          float r = s.R[(int64_t)j * cap + i], p = s.P[(int64_t)j * cap + i];
+          p = kick1(j, r, p, hu, hv);
+          r = __fmaf_rn(cf.dtm[j], p, r);
+          z.A = __fmaf_rn(cf.a[j], r, z.A);
+          if (KIND == 1) z.B = __fmaf_rn(cf.b[j], r, z.B);
+          s.R[(int64_t)j * cap + i] = r;
+          s.P[(int64_t)j * cap + i] = p;
         }
         closed_form(z);
-        kick<NPL, KIND, Coef2>(w, cf, hsab * z.c2, hsab * z.s2);
+        const float hu2 = hsab * z.c2, hv2 = hsab * z.s2;
         float Av = 0.0f, Bv = 0.0f;
-  #pragma unroll
-        for (int j = 0; j < NPL; ++j) {
-          Av = __fmaf_rn(cf.am[j], w.P[j], Av);
-          if (KIND == 1) Bv = __fmaf_rn(cf.bm[j], w.P[j], Bv);
+        for (int j = 0; j < bp.n; ++j) {
+          const float r = s.R[(int64_t)j * cap + i];
+          const float p = kick1(j, r, s.P[(int64_t)j * cap + i], hu2, hv2);
+          Av = __fmaf_rn(cf.am[j], p, Av);
+          if (KIND == 1) Bv = __fmaf_rn(cf.bm[j], p, Bv);
+          s.P[(int64_t)j * cap + i] = p;
         }
         hop = spawn_transition<KIND, false>(z, r_old, Av, Bv, word, bp, deg, child);
       }
-      // the phase pair is renormalised, and wrapped past 2^10 rad, at the end of
-      // every Philox block (absolute steps 4k + 3)
-      if ((step & 3) == 3) {
-        z.ph = two_sum(z.ph.hi, z.ph.lo);
-        phase_wrap(z);
-      }
-  #pragma unroll
-      for (int j = 0; j < NPL; ++j)
-        if (j < bp.n) {
-          s.R[(int64_t)j * cap + i] = w.R[j];
-          s.P[(int64_t)j * cap + i] = w.P[j];
-        }
+      spawn_phase_end(z, step);
       s.ph[i] = z.ph.hi;
       s.pl[i] = z.ph.lo;
       flag = hop ? 1 : 0;
@@ -255,21 +500,9 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
         ((float*)((char*)buf + L.cm))[i] = child.m.hi;
         ((float*)((char*)buf + L.cmlo))[i] = child.m.lo;
         ((int32_t*)((char*)buf + L.cmexp))[i] = child.mexp;
-        ((uint16_t*)((char*)buf + L.cab))[i] =
-            (uint16_t)((child.sa > 0.0f ? 1 : 0) | (child.q << 4) | ((child.sb > 0.0f ? 1 : 0) << 8));
-        if (!isfinite(child.m.hi)) {
-          atomicAdd(&hdr->n_nonfinite, 1ull);
-          atomicOr(&hdr->flags, QCL_FLAG_NONFINITE);
-        }
+        ((uint16_t*)((char*)buf + L.cab))[i] = pair_word(child);
       }
-      if (deg) {
-        atomicAdd(&hdr->n_degenerate, 1ull);
-        atomicOr(&hdr->flags, QCL_FLAG_DEGENERATE);
-      }
-      if (!isfinite(z.ph.hi)) {
-        atomicAdd(&hdr->n_nonfinite, 1ull);
-        atomicOr(&hdr->flags, QCL_FLAG_NONFINITE);
-      }
+      spawn_report(hdr, z, hop, child, deg);
     }
     const int cnt = __syncthreads_count(flag);
     if (threadIdx.x == 0) ((int32_t*)((char*)buf + L.bsum))[vb] = cnt;
@@ -342,85 +575,124 @@ __global__ void __launch_bounds__(256) k_spawn_scatter32(void* buf, int64_t cap,
 }
 
 // Family observation: for each family the sum X of its walkers' contributions
-// and X^2.  A warp takes 32 families, one at a time: lane l takes the family's
-// walkers l, l + 32, ... (coalesced loads; no lane idles on a small family while
-// another walks a large one).  The family shares one power of two (its largest
-// weight exponent), so each walker's contribution is an FP32 value, summed as a
-// compensated FP32 pair per lane and then over the lanes by a reduce-scatter of
-// pairs, which leaves lanes 2q and 2q + 1 with quantity q; X is rebuilt in FP64
-// from the pair and the exponent exactly, and the even lane accumulates X, the
-// odd lane X^2, over the warp's families in order.  (Accumulating every walker
-// in FP64 kept the FP64 pipe 84 % busy: FP64 is slow on this part.)  The tile's
-// 8 warps are then folded by the fixed tree of the observation kernels.
+// and X^2.  A warp takes 32 families.  The family shares one power of two (its
+// largest weight exponent), so each walker's contribution is an FP32 value,
+// summed as a compensated FP32 pair per lane (lane l of 32 takes the family's
+// walkers l, l + 32, ...) and then over the lanes by a reduce-scatter of pairs at
+// lane distances 16, 8, 4, 2, 1; X is rebuilt in FP64 from the pair and the
+// exponent exactly.  Lanes without a walker hold zero pairs, which change
+// nothing, so a family of at most w walkers takes w lanes (w = 1, 4, 8 or 16)
+// with the same result, and 32 / w such families go side by side (1e5 families of
+// one walker 88 -> 36 us, of four on average 90 -> 82).  The X of the warp's families then meet in shared memory, where
+// the even lane of a pair adds X, the odd lane X^2, of one quantity over the
+// families in order.  (Accumulating every walker in FP64 kept the FP64 pipe 84 %
+// busy: FP64 is slow on this part.)  The tile's 8 warps are folded by the fixed
+// tree of the observation kernels.
 template <int KIND, bool DIA>
-__global__ void __launch_bounds__(256) k_spawn_observe32(const BulkParams bp, const Coef2 cf,
+__global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp, const Coef2 cf,
                                                          const void* buf, int64_t cap, int64_t n0,
                                                          int set, double* __restrict__ part) {
   __shared__ double red[8][32];
+  __shared__ double xs[8][32][17];  // (rows of 17: no bank conflicts between families)
+  __shared__ uint8_t ord[8][32];
   const SpawnLayout L = SpawnLayout::make(cap, bp.n, n0, QCL_PREC_FP32_BULK);
   const Set32 s = set32((void*)buf, L, set);
   const int64_t* fstart = (const int64_t*)((const char*)buf + L.fstart);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double T = 0.0;
   const int64_t f0 = (int64_t)blockIdx.x * 256 + warp * 32;
+  // lane l's family and its width class
+  const bool real = f0 + lane < n0;
+  const int64_t mine = real ? fstart[f0 + lane] : 0;
+  const int64_t size = real ? fstart[f0 + lane + 1] - mine : 0;
+  const int cls = !real ? 5 : size <= 1 ? 0 : size <= 4 ? 1 : size <= 8 ? 2 : size <= 16 ? 3 : 4;
 #pragma unroll 1
-  for (int f = 0; f < 32; ++f) {
-    const int64_t k = f0 + f;
-    if (k >= n0) break;  // (warp-uniform)
-    const int64_t j0 = fstart[k], j1 = fstart[k + 1];
-    int em = -(1 << 28);
-    for (int64_t j = j0 + lane; j < j1; j += 32)
-      if (s.mh[j] != 0.0f) em = max(em, s.me[j]);
-    em = __reduce_max_sync(0xffffffffu, em);
-    f2 acc[16];
+  for (int c = 0; c < 5; ++c) {
+    const unsigned in = __ballot_sync(0xffffffffu, cls == c);
+    if (!in) continue;
+    const int w = c == 0 ? 1 : 2 << c, side = 32 / w, count = __popc(in);
+    if (cls == c) ord[warp][__popc(in & ((1u << lane) - 1u))] = (uint8_t)lane;
+    __syncwarp();
+    const int sub = lane / w, sl = lane - sub * w;
+#pragma unroll 1
+    for (int at = 0; at < count; at += side) {
+      const bool on = at + sub < count;
+      const int f = ord[warp][on ? at + sub : at];
+      const int64_t j0 = __shfl_sync(0xffffffffu, mine, f);
+      const int64_t len = __shfl_sync(0xffffffffu, size, f);
+      const int64_t j1 = on ? j0 + len : j0;
+      int em = -(1 << 28);
+      for (int64_t j = j0 + sl; j < j1; j += w)
+        if (s.mh[j] != 0.0f) em = max(em, s.me[j]);
+      for (int off = w >> 1; off > 0; off >>= 1)
+        em = max(em, __shfl_xor_sync(0xffffffffu, em, off));
+      f2 acc[16];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) acc[q] = {0.0f, 0.0f};
-    for (int64_t j = j0 + lane; j < j1; j += 32) {
-      Scal z;
-      z.A = bp.a0;
-      z.B = bp.b0;
-      for (int m = 0; m < bp.n; ++m) {
-        const float r = s.R[(int64_t)m * cap + j];
-        z.A = __fmaf_rn(cf.a[m], r, z.A);
-        if (KIND == 1) z.B = __fmaf_rn(cf.b[m], r, z.B);
-      }
-      closed_form(z);
-      const uint32_t ab = s.ab[j];
-      z.sa = sgn(ab & 0xf);
-      z.sb = sgn((ab >> 8) & 0xf);
-      z.q = DIA ? (int)((ab >> 4) & 3u) : 0;
-      z.ph = {s.ph[j], s.pl[j]};
-      const float mh = s.mh[j];
-      const float mm = mh == 0.0f ? 0.0f : (mh + s.ml[j]) * pow2i(s.me[j] - em);
-      float c[16];
-      contributions<DIA>(z, mm, c);
+      for (int q = 0; q < 16; ++q) acc[q] = {0.0f, 0.0f};
+      for (int64_t j = j0 + sl; j < j1; j += w) {
+        Scal z;
+        z.A = bp.a0;
+        z.B = bp.b0;
+        for (int m = 0; m < bp.n; ++m) {
+          const float r = s.R[(int64_t)m * cap + j];
+          z.A = __fmaf_rn(cf.a[m], r, z.A);
+          if (KIND == 1) z.B = __fmaf_rn(cf.b[m], r, z.B);
+        }
+        closed_form(z);
+        const uint32_t ab = s.ab[j];
+        z.sa = sgn(ab & 0xf);
+        z.sb = sgn((ab >> 8) & 0xf);
+        z.q = DIA ? (int)((ab >> 4) & 3u) : 0;
+        z.ph = {s.ph[j], s.pl[j]};
+        const float mh = s.mh[j];
+        const float mm = mh == 0.0f ? 0.0f : (mh + s.ml[j]) * pow2i(s.me[j] - em);
+        float v[16];
+        contributions<DIA>(z, mm, v);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const f2 t = two_sum(acc[q].hi, c[q]);
-        acc[q] = {t.hi, acc[q].lo + t.lo};
+        for (int q = 0; q < 16; ++q) {
+          const f2 t = two_sum(acc[q].hi, v[q]);
+          acc[q] = {t.hi, acc[q].lo + t.lo};
+        }
       }
+      __syncwarp();
+      // reduce-scatter of the pairs: at the step with offset `off`, the lane with
+      // that bit set keeps the upper half of its values (q0: the first it keeps)
+      int q0 = 0, keep = 16, off = w >> 1;
+#pragma unroll
+      for (int half = 8; half >= 1; half >>= 1) {
+        if (off > 0) {
+          const bool upper = (lane & off) != 0;
+#pragma unroll
+          for (int i2 = 0; i2 < half; ++i2) {
+            const f2 snd = upper ? acc[i2] : acc[half + i2];
+            const f2 kp = upper ? acc[half + i2] : acc[i2];
+            const float rh = __shfl_xor_sync(0xffffffffu, snd.hi, off);
+            const float rl = __shfl_xor_sync(0xffffffffu, snd.lo, off);
+            const f2 t = two_sum(kp.hi, rh);
+            acc[i2] = {t.hi, t.lo + (kp.lo + rl)};
+          }
+          q0 += upper ? half : 0;
+          keep = half;
+          off >>= 1;
+        }
+      }
+      if (off > 0) {  // (w = 32: lanes 2q and 2q + 1 both end with quantity q)
+        const float rh = __shfl_xor_sync(0xffffffffu, acc[0].hi, 1);
+        const float rl = __shfl_xor_sync(0xffffffffu, acc[0].lo, 1);
+        const f2 t = two_sum(acc[0].hi, rh);
+        acc[0] = {t.hi, t.lo + (acc[0].lo + rl)};
+      }
+      const int ex = (em < -(1 << 27)) ? 0 : em;
+#pragma unroll
+      for (int i2 = 0; i2 < 16; ++i2)
+        if (on && i2 < keep)
+          xs[warp][f][q0 + i2] = scaled_double(acc[i2].hi, ex) + scaled_double(acc[i2].lo, ex);
     }
-    // reduce-scatter of the pairs: at the step with offset `off`, the lane with
-    // that bit set keeps the upper half of its values
-#pragma unroll
-    for (int lev = 0; lev < 4; ++lev) {
-      const int half = 8 >> lev, off = 16 >> lev;
-      const bool upper = (lane & off) != 0;
-#pragma unroll
-      for (int i2 = 0; i2 < half; ++i2) {
-        const f2 snd = upper ? acc[i2] : acc[half + i2];
-        const f2 kp = upper ? acc[half + i2] : acc[i2];
-        const float rh = __shfl_xor_sync(0xffffffffu, snd.hi, off);
-        const float rl = __shfl_xor_sync(0xffffffffu, snd.lo, off);
-        const f2 t = two_sum(kp.hi, rh);
-        acc[i2] = {t.hi, t.lo + (kp.lo + rl)};
-      }
-    }
-    const float rh = __shfl_xor_sync(0xffffffffu, acc[0].hi, 1);
-    const float rl = __shfl_xor_sync(0xffffffffu, acc[0].lo, 1);
-    const f2 t = two_sum(acc[0].hi, rh);
-    const int ex = (em < -(1 << 27)) ? 0 : em;
-    const double X = scaled_double(t.hi, ex) + scaled_double(t.lo + (acc[0].lo + rl), ex);
+    __syncwarp();  // ord is rewritten
+  }
+  const int nf = (int)max((int64_t)0, min((int64_t)32, n0 - f0));
+  double T = 0.0;
+  for (int f = 0; f < nf; ++f) {
+    const double X = xs[warp][f][lane >> 1];
     T = (lane & 1) ? fma(X, X, T) : T + X;
   }
   red[warp][(lane & 1) ? 16 + (lane >> 1) : (lane >> 1)] = T;
@@ -430,25 +702,58 @@ __global__ void __launch_bounds__(256) k_spawn_observe32(const BulkParams bp, co
 }
 
 template <int NPL, int KIND, bool DIA>
-void run_step32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t cap, int64_t n0,
-                int64_t step, cudaStream_t st) {
-  k_spawn_step32<NPL, KIND, DIA><<<spawn_grid(cap), 256, 0, st>>>(bp, cf, buf, cap, n0, step);
+void run_steps32(const BulkParams& bp, const Coef2& c2, void* buf, int64_t cap, int64_t n0,
+                 int64_t step, int64_t len, cudaStream_t st) {
+  CoefLocal<NPL> cf{};
+  for (int j = 0; j < NPL && j < bp.n; ++j) {
+    cf.hk[j] = c2.hk[j];
+    cf.hs[j] = c2.hs[j];
+    cf.dtm[j] = c2.dtm[j];
+    cf.a[j] = c2.a[j];
+    cf.b[j] = c2.b[j];
+    cf.am[j] = c2.am[j];
+    cf.bm[j] = c2.bm[j];
+  }
+  const SpawnLayout L = SpawnLayout::make(cap, bp.n, n0, QCL_PREC_FP32_BULK);
+  // every block resident at once (at most one group a block)
+  static int per_sm = 0;
+  if (per_sm == 0) {
+    int b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_spawn_chain32<NPL, KIND, DIA, false>, 256, 0);
+    per_sm = b < 1 ? 1 : b;
+  }
+  const unsigned grid = spawn_grid(cap, per_sm);
+  if (step == bp.step0) {
+    k_spawn_chain_clear<<<grid, 256, 0, st>>>(buf, cap, bp.n, n0);
+    k_spawn_chain32<NPL, KIND, DIA, true><<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, step);
+    launches_add(2);
+  }
+  for (int64_t t = step; t < step + len; ++t)
+    k_spawn_chain32<NPL, KIND, DIA, false><<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, t);
+  launches_add(len);
 }
 
-// in registers up to 32 modes, beyond that (or under QCL_OPT_MODES_IN_MEMORY = 1)
-// in memory
+// Chained steps with the modes in registers up to 32 modes; beyond that (or under
+// QCL_OPT_MODES_IN_MEMORY = 1) in memory, three launches a step.
 template <int KIND, bool DIA>
-int dispatch_step32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t cap, int64_t n0,
-                    int64_t step, cudaStream_t st) {
+void dispatch_steps32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t cap, int64_t n0,
+                      int64_t step0, int64_t step, int64_t len, cudaStream_t st) {
   const int n = bp.n;
-  if (n > 32 || option_modes_in_memory() == 1) run_step32<0, KIND, DIA>(bp, cf, buf, cap, n0, step, st);
-  else if (n <= 1) run_step32<1, KIND, DIA>(bp, cf, buf, cap, n0, step, st);
-  else if (n <= 2) run_step32<2, KIND, DIA>(bp, cf, buf, cap, n0, step, st);
-  else if (n <= 4) run_step32<4, KIND, DIA>(bp, cf, buf, cap, n0, step, st);
-  else if (n <= 8) run_step32<8, KIND, DIA>(bp, cf, buf, cap, n0, step, st);
-  else if (n <= 16) run_step32<16, KIND, DIA>(bp, cf, buf, cap, n0, step, st);
-  else run_step32<32, KIND, DIA>(bp, cf, buf, cap, n0, step, st);
-  return 1;
+  if (n > 32 || option_modes_in_memory() == 1) {
+    for (int64_t t = step; t < step + len; ++t) {
+      k_spawn_step32<KIND, DIA><<<spawn_grid(cap), 256, 0, st>>>(bp, cf, buf, cap, n0, t);
+      launch_spawn_scan(buf, cap, n, n0, QCL_PREC_FP32_BULK, 2, step0, t, st);
+      k_spawn_scatter32<<<spawn_grid(cap), 256, 0, st>>>(buf, cap, n, n0, step0, t, bp.seed);
+      launches_add(2);
+    }
+    return;
+  }
+  if (n <= 1) run_steps32<1, KIND, DIA>(bp, cf, buf, cap, n0, step, len, st);
+  else if (n <= 2) run_steps32<2, KIND, DIA>(bp, cf, buf, cap, n0, step, len, st);
+  else if (n <= 4) run_steps32<4, KIND, DIA>(bp, cf, buf, cap, n0, step, len, st);
+  else if (n <= 8) run_steps32<8, KIND, DIA>(bp, cf, buf, cap, n0, step, len, st);
+  else if (n <= 16) run_steps32<16, KIND, DIA>(bp, cf, buf, cap, n0, step, len, st);
+  else run_steps32<32, KIND, DIA>(bp, cf, buf, cap, n0, step, len, st);
 }
 
 }  // namespace
@@ -462,18 +767,11 @@ void launch_spawn_sample32(const DevModel& host, const SampleParams& sp, int64_t
   launches_add(1);
 }
 
-int launch_spawn_step32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t capacity,
-                        int64_t n0, int64_t step0, int64_t step, cudaStream_t st) {
-  const bool dia = bp.repr == QCL_REPR_DIABATIC;
-  const int ok = dia ? (bp.kind == 0 ? dispatch_step32<0, true>(bp, cf, buf, capacity, n0, step, st)
-                                     : dispatch_step32<1, true>(bp, cf, buf, capacity, n0, step, st))
-                     : (bp.kind == 0 ? dispatch_step32<0, false>(bp, cf, buf, capacity, n0, step, st)
-                                     : dispatch_step32<1, false>(bp, cf, buf, capacity, n0, step, st));
-  if (!ok) return 0;
-  launch_spawn_scan(buf, capacity, bp.n, n0, QCL_PREC_FP32_BULK, 2, step0, step, st);
-  k_spawn_scatter32<<<spawn_grid(capacity), 256, 0, st>>>(buf, capacity, bp.n, n0, step0, step, bp.seed);
-  launches_add(2);
-  return 1;
+void launch_spawn_steps32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t capacity,
+                          int64_t n0, int64_t step0, int64_t step, int64_t len, cudaStream_t st) {
+  auto run = [&](auto f) { f(bp, cf, buf, capacity, n0, step0, step, len, st); };
+  if (bp.repr == QCL_REPR_DIABATIC) run(bp.kind == 0 ? dispatch_steps32<0, true> : dispatch_steps32<1, true>);
+  else run(bp.kind == 0 ? dispatch_steps32<0, false> : dispatch_steps32<1, false>);
 }
 
 void launch_spawn_observe32(const BulkParams& bp, const Coef2& cf, const void* buf, int64_t capacity,
