@@ -51,29 +51,6 @@ __device__ __forceinline__ void half_angle(const Ad2& d, double& c, double& s) {
   }
 }
 
-// The decomposition at R read from the SoA arrays (stride nt).
-__device__ __forceinline__ Ad2 decomp_g(const DevModel* M, const double* R, int64_t nt, int n) {
-  double a = M->a0, b = M->b0;
-  for (int j = 0; j < n; ++j) {
-    const double x = R[(int64_t)j * nt];
-    a += M->a[j] * x;
-    b += M->b[j] * x;
-  }
-  Ad2 d;
-  d.a = a;
-  d.b = b;
-  d.r = sqrt(a * a + b * b);
-  if (d.r > 0.0) {
-    d.c2 = a / d.r;
-    d.s2 = b / d.r;
-  } else {
-    d.c2 = 1.0;
-    d.s2 = 0.0;
-  }
-  return d;
-}
-
-
 template <typename T>
 __device__ __forceinline__ void pick_pair(const double* rho_ad, int ns, uint32_t word,
                                           int& al, int& be, double& m0) {
@@ -452,40 +429,48 @@ inline void dispatch_f64(const DevModel& h, F&& f) {
   else np(std::integral_constant<int, 0>{});
 }
 
-// The 16 observable contributions of one walker and their squares (v[16..31]):
-// z = m exp(-i phi) i^q at the walker's own pair in its own representation,
-// z U_ia U_jb (U symmetric) at every element of the other.  R at Rg[j * stride].
-__device__ __forceinline__ void contrib_f64(const DevModel* __restrict__ M, const double* Rg,
-                                            int64_t stride, int n, double m, double phi,
-                                            uint16_t ab, double (&v)[32]) {
-  const Ad2 d = decomp_g(M, Rg, stride, n);
-  double c, s;
-  half_angle(d, c, s);
-  const double U[4] = {-s, c, c, s};
+// The 16 observable contributions of one walker and their squares (v[16..31])
+// from the decomposition at its R (of the adiabatic form): z = m exp(-i phi) i^q
+// at the walker's own pair in its own representation, z U_ia U_jb (U symmetric) at
+// every element of the other.  The eigenvector angle by the cancellation-free
+// half-angle form: the larger of cos, sin theta is sqrt((1 + |cos 2theta|) / 2).
+__device__ __forceinline__ void contrib_f64(const Dec64& d, double m, double phi, uint16_t ab,
+                                            bool dia, double (&v)[32]) {
+  double s2 = __dmul_rn(d.b, __dmul_rn(d.r, d.ir2));
+  if (d.deg) s2 = d.r > 0.0 ? d.b / d.r : 0.0;
+  const double t = __fma_rn(0.5, fabs(d.c2), 0.5);
+  const double rt = rsqrt64(t);
+  const double big = __dmul_rn(t, rt), small = __dmul_rn(__dmul_rn(0.5, fabs(s2)), rt);
+  const bool cpos = d.c2 >= 0.0;
+  const double c = cpos ? big : small;
+  const double s = copysign(cpos ? small : big, s2);
   const int al = ab & 0xf, be = (ab >> 8) & 0xf, q = (ab >> 4) & 3;
   double sn, cs;
   sincos(phi, &sn, &cs);
-  const double xr = m * cs, xi = -m * sn;
+  const double xr = __dmul_rn(m, cs), xi = -__dmul_rn(m, sn);
   const double zr = q == 0 ? xr : (q == 1 ? -xi : (q == 2 ? -xr : xi));
   const double zi = q == 0 ? xi : (q == 1 ? xr : (q == 2 ? -xi : -xr));
-  const bool dia = M->repr == QCL_REPR_DIABATIC;
-  const int own = dia ? 0 : 8, other = dia ? 8 : 0;
-#pragma unroll
-  for (int ii = 0; ii < 2; ++ii)
-#pragma unroll
-    for (int jj = 0; jj < 2; ++jj) {
-      const double f = U[ii * 2 + al] * U[jj * 2 + be];
-      v[other + 2 * (ii * 2 + jj)] = zr * f;
-      v[other + 2 * (ii * 2 + jj) + 1] = zi * f;
-    }
+  const double r2 = __dmul_rn(zr, zr), i2 = __dmul_rn(zi, zi);
+  const double ua[2] = {al ? c : -s, al ? s : c}, ub[2] = {be ? c : -s, be ? s : c};
+  const int k0 = al * 2 + be;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const bool hit = (k == al * 2 + be);
-    v[own + 2 * k] = hit ? zr : 0.0;
-    v[own + 2 * k + 1] = hit ? zi : 0.0;
+    const double f = __dmul_rn(ua[k >> 1], ub[k & 1]);
+    const double fr = __dmul_rn(zr, f), fi = __dmul_rn(zi, f);
+    const double fr2 = __dmul_rn(fr, fr), fi2 = __dmul_rn(fi, fi);
+    const bool hit = k == k0;
+    const double hr = hit ? zr : 0.0, hi = hit ? zi : 0.0;
+    const double hr2 = hit ? r2 : 0.0, hi2 = hit ? i2 : 0.0;
+    // (the diabatic block first, the adiabatic one after it)
+    v[2 * k] = dia ? hr : fr;
+    v[2 * k + 1] = dia ? hi : fi;
+    v[8 + 2 * k] = dia ? fr : hr;
+    v[8 + 2 * k + 1] = dia ? fi : hi;
+    v[16 + 2 * k] = dia ? hr2 : fr2;
+    v[16 + 2 * k + 1] = dia ? hi2 : fi2;
+    v[24 + 2 * k] = dia ? fr2 : hr2;
+    v[24 + 2 * k + 1] = dia ? fi2 : hi2;
   }
-#pragma unroll
-  for (int q2 = 0; q2 < 16; ++q2) v[16 + q2] = v[q2] * v[q2];
 }
 
 }  // namespace qcl

@@ -362,11 +362,11 @@ void launches_add(int64_t k);
 int64_t launches_read(bool reset);
 
 void launch_sample_f64(const DevModel* dm, const SampleParams& sp, void* buf, cudaStream_t st);
-// Steps [step, step + len) of a two-state ensemble (one launch).
-void launch_steps_f64(const DevModel& host, void* buf, int64_t nt, int64_t step0, int64_t step,
-                      int32_t len, double dt, uint64_t seed, uint64_t traj_off, cudaStream_t st);
-void launch_observe_f64(const DevModel* dm, const void* buf, int64_t nt, int n, double* part,
-                        cudaStream_t st);
+// Steps of a two-state ensemble from `step` towards `end` with their output
+// times, one launch and one fold to tiles (kernels_f64.cu).
+int64_t launch_steps_f64(const DevModel& host, void* buf, int64_t nt, int64_t step0, int64_t step,
+                         int64_t end, int32_t stride, bool obs_first, double dt, uint64_t seed,
+                         uint64_t traj_off, double* part, int* outs, cudaStream_t st);
 
 // Launch shape of a persistent bulk launch; the results do not depend on it.
 struct LaunchShape {

@@ -486,29 +486,33 @@ qcl_status qcl_propagate(const qcl_model* model, const qcl_ensemble_desc* ens, v
 
   if (ens->precision == QCL_PREC_FP64) {
     const int ns = model->ns;
-    auto observe = [&](int64_t k) {
-      if (ns == 2)
-        launch_observe_f64(model->dev, ens_buf, nt, model->n, part, s);
-      else
-        launch_observeN_f64(model->dev, ns, ens_buf, nt, model->n, part, s);
-      launch_fold(part, rows + (size_t)k * q2, fold, OL.n_tiles, q2, 1, s, chunk_row(k));
-    };
-    if (step0 == 0) observe(0);
     const int64_t end = step0 + n_steps;
-    for (int64_t t = step0; t < end;) {
-      // two states: up to the next output time in one launch, at most 256 steps
-      // (a launch of 1e7 walkers then stays below a second); more states: one step
-      int64_t len = 1;
-      if (ns == 2) len = std::min<int64_t>(std::min<int64_t>(end, (t / out_stride + 1) * out_stride) - t, 256);
-      {
-        TimedLaunch tl(1, s);
-        if (ns == 2)
-          launch_steps_f64(model->host, ens_buf, nt, step0, t, (int32_t)len, dt, ens->seed, ens->traj_id_offset, s);
-        else
-          launch_stepN_f64(model->dev, model->host.repr, ns, ens_buf, nt, model->n, step0, t, dt, ens->seed, ens->traj_id_offset, s);
+    if (ns == 2) {
+      bool first = step0 == 0;
+      for (int64_t t = step0; t < end || first;) {
+        const int64_t k_first = first ? 0 : t / out_stride + 1;
+        int outs = 0;
+        {
+          TimedLaunch tl(1, s);
+          t += launch_steps_f64(model->host, ens_buf, nt, step0, t, end, out_stride, first, dt, ens->seed,
+                                ens->traj_id_offset, part, &outs, s);
+        }
+        if (outs > 0) launch_fold(part, rows + (size_t)k_first * q2, fold, OL.n_tiles, q2, outs, s, chunk_row(k_first));
+        first = false;
       }
-      t += len;
-      if (t % out_stride == 0) observe(t / out_stride);
+    } else {
+      auto observe = [&](int64_t k) {
+        launch_observeN_f64(model->dev, ns, ens_buf, nt, model->n, part, s);
+        launch_fold(part, rows + (size_t)k * q2, fold, OL.n_tiles, q2, 1, s, chunk_row(k));
+      };
+      if (step0 == 0) observe(0);
+      for (int64_t t = step0; t < end; ++t) {
+        {
+          TimedLaunch tl(1, s);
+          launch_stepN_f64(model->dev, model->host.repr, ns, ens_buf, nt, model->n, step0, t, dt, ens->seed, ens->traj_id_offset, s);
+        }
+        if ((t + 1) % out_stride == 0) observe((t + 1) / out_stride);
+      }
     }
     st = check_launch("FP64 step");
     if (st) return st;

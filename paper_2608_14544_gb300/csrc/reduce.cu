@@ -27,6 +27,8 @@ __global__ void __launch_bounds__(256) k_fold_level(const double* __restrict__ i
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int64_t base = blk * 1024 + (int64_t)(w * 4 + k) * 32;
+    g[k] = 0.0;
+    if (base >= n) continue;  // (zero leaves add nothing: 1e4 walkers have 40 tiles)
     double v[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) {

@@ -295,7 +295,16 @@ __global__ void __launch_bounds__(256) k_spawn_observe(const DevModel* __restric
     const int64_t j0 = fstart[k], j1 = fstart[k + 1];
     for (int64_t j = j0; j < j1; ++j) {
       double c[32];
-      contrib_f64(M, s.R + j, cap, n, s.m[j], s.phi[j], s.ab[j], c);
+      Dec64 d;
+      d.a = M->a0;
+      d.b = M->b0;
+      for (int k2 = 0; k2 < n; ++k2) {
+        const double x = s.R[(int64_t)k2 * cap + j];
+        d.a = __fma_rn(M->a[k2], x, d.a);
+        d.b = __fma_rn(M->b[k2], x, d.b);
+      }
+      decompose64<0, false>(d);
+      contrib_f64(d, s.m[j], s.phi[j], s.ab[j], M->repr == QCL_REPR_DIABATIC, c);
 #pragma unroll
       for (int q = 0; q < 16; ++q) v[q] += c[q];
     }
