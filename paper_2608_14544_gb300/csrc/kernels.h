@@ -414,9 +414,10 @@ const char* bulk2_variant(int n, int kind);
 // N_s-state initial sample: FP64 (dm, sp) or FP32 bulk (s32).
 void launch_sampleN(const DevModel* dm, const SampleParams& sp, const SampleN32* s32, void* buf,
                     int precision, cudaStream_t st);
-void launch_stepN_f64(const DevModel* dm, int repr, int ns, void* buf, int64_t nt, int n,
-                      int64_t step0, int64_t step, double dt, uint64_t seed, uint64_t traj_off,
-                      cudaStream_t st);
+// Steps [step, step + len) of an N_s-state ensemble (one launch).
+void launch_stepsN_f64(const DevModel* dm, int repr, int ns, void* buf, int64_t nt, int n,
+                       int64_t step0, int64_t step, int32_t len, double dt, uint64_t seed,
+                       uint64_t traj_off, cudaStream_t st);
 void launch_observeN_f64(const DevModel* dm, int ns, const void* buf, int64_t nt, int n,
                          double* part, cudaStream_t st);
 int launch_bulkN(int ns, const BulkParams& bp, const CoefN& cf, const ModeHost& mh, void* buf,

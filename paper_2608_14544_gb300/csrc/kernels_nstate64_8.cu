@@ -7,8 +7,9 @@ void nstate_sample64_8(const DevModel* dm, const SampleParams& sp, void* buf, cu
   NStateOps<8>::sample64(dm, sp, buf, st);
 }
 void nstate_step64_8(const DevModel* dm, int repr, void* buf, int64_t nt, int n, int64_t step0,
-                     int64_t step, double dt, uint64_t seed, uint64_t traj_off, cudaStream_t st) {
-  NStateOps<8>::step64(dm, repr, buf, nt, n, step0, step, dt, seed, traj_off, st);
+                     int64_t step, int32_t len, double dt, uint64_t seed, uint64_t traj_off,
+                     cudaStream_t st) {
+  NStateOps<8>::step64(dm, repr, buf, nt, n, step0, step, len, dt, seed, traj_off, st);
 }
 void nstate_spawn_sample64_8(const DevModel* dm, const SampleParams& sp, int64_t cap, void* buf,
                              cudaStream_t st) {

@@ -1,5 +1,5 @@
 // nstate_f64.cuh -- the FP64 path of N_s-state models: sampling, one launch
-// per step (adiabatic and diabatic), observation and trajectory spawning, in
+// per output time (adiabatic and diabatic), observation and trajectory spawning, in
 // the oracle's operation order (its units are compiled without multiply-add
 // contraction).
 #pragma once
@@ -148,24 +148,30 @@ __device__ __forceinline__ StepN draw_event(const double (&A)[NC], const uint64_
   return {hit, Ah, Th, sumT, deg};
 }
 
+// The decomposition at a walker's R, gauge following the eigenvectors ref.
+template <int NS>
+__device__ __forceinline__ void decompose_ref_f64(const DevModel* __restrict__ M, const double* R,
+                                                  int64_t nt, int n, const double (&ref)[NS][NS],
+                                                  double (&e)[NS], double (&U)[NS][NS]) {
+  double W[NS][NS];
+  elec_g<NS>(M, R, nt, n, W);
+  eigh_ns<double, NS>(W, ref, e, U, 100, 1e-34, false);
+}
+
 // Adiabatic pairs: velocity Verlet on the pair's mean force with the
-// decompositions at R_n and R_{n+1} (gauge following the carried eigenvectors
-// Uc; U1 receives those at R_{n+1}), the trapezoid phase, the 2 N_s event
-// slots' amplitudes and thresholds, and the draw.  R and P at R[j * nt].
+// decompositions at R_n (e0, U0) and R_{n+1} (gauge following U0; e1, U1 receive
+// it), the trapezoid phase, the 2 N_s event slots' amplitudes and thresholds,
+// and the draw.  R and P at R[j * nt].
 template <int NS>
 __device__ __forceinline__ StepN walker_stepN_f64(const DevModel* __restrict__ M, double* R,
                                                   double* P, int64_t nt, int n, int al, int be,
-                                                  double& phi, const double (&Uc)[NS][NS],
+                                                  double& phi, const double (&e0)[NS],
+                                                  const double (&U0)[NS][NS], double (&e1)[NS],
                                                   double (&U1)[NS][NS], double dt, uint64_t seed,
                                                   uint64_t traj, int64_t step) {
-  double W[NS][NS], e0[NS], U0[NS][NS], e1[NS];
-  // decomposition at R_n, gauge following the carried eigenvectors
-  elec_g<NS>(M, R, nt, n, W);
-  eigh_ns<double, NS>(W, Uc, e0, U0, 100, 1e-34, false);
   half_kick_g<NS>(M, R, P, nt, n, U0, al, be, dt);
   for (int j = 0; j < n; ++j) R[(int64_t)j * nt] += dt * P[(int64_t)j * nt] / M->mass[j];
-  elec_g<NS>(M, R, nt, n, W);
-  eigh_ns<double, NS>(W, U0, e1, U1, 100, 1e-34, false);
+  decompose_ref_f64<NS>(M, R, nt, n, U0, e1, U1);
   half_kick_g<NS>(M, R, P, nt, n, U1, al, be, dt);
   const double w0 = (pick<double, NS>(e0, al) - pick<double, NS>(e0, be)) / M->hbar;
   const double w1 = (pick<double, NS>(e1, al) - pick<double, NS>(e1, be)) / M->hbar;
@@ -240,10 +246,18 @@ __device__ __forceinline__ StepN walker_stepN_f64(const DevModel* __restrict__ M
   return draw_event<NC>(A, T, sumT, deg, seed, traj, step);
 }
 
+// `len` steps of one walker per thread.  The decomposition at R_{n+1} is the next
+// step's at R_n: a cold decomposition of the same matrix, whose gauge follows the
+// same eigenvectors, gives the same bits, so it is carried and only the first
+// step of a launch makes it afresh (10.9 thousand FP64 instructions a walker-step
+// of the four-state six-mode model with both, 7.4 thousand with one).  Bound by the
+// FP64 unit; blocks of one warp, so that 2e4 walkers spread evenly over the SMs
+// (157 blocks of 128 left five of 152 SMs with two).
 template <int NS>
-__global__ void __launch_bounds__(128) k_stepN_f64(const DevModel* __restrict__ M, void* buf,
+__global__ void __launch_bounds__(32) k_stepsN_f64(const DevModel* __restrict__ M, void* buf,
                                                    int64_t nt, int n, int64_t step0, int64_t step,
-                                                   double dt, uint64_t seed, uint64_t traj_off) {
+                                                   int32_t len, double dt, uint64_t seed,
+                                                   uint64_t traj_off) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   WN<double> w = viewN<double>(buf, nt, NS, n, QCL_PREC_FP64);
   if (i >= nt) return;
@@ -254,19 +268,36 @@ __global__ void __launch_bounds__(128) k_stepN_f64(const DevModel* __restrict__ 
   const uint16_t ab = w.ab[i];
   int al = ab & 0xf, be = (ab >> 8) & 0xf;
   double m = w.m[i], phi = w.phi[i];
-  double Uc[NS][NS], U1[NS][NS];
+  double e0[NS], U0[NS][NS];
+  {
+    double Uc[NS][NS];
 #pragma unroll
-  for (int a = 0; a < NS; ++a)
+    for (int a = 0; a < NS; ++a)
 #pragma unroll
-    for (int b = 0; b < NS; ++b) Uc[a][b] = w.U[(int64_t)(a * NS + b) * nt + i];
-  const StepN o = walker_stepN_f64<NS>(M, w.R + i, w.P + i, nt, n, al, be, phi, Uc, U1, dt, seed,
-                                       traj_off + (uint64_t)i, step);
-  if (o.hit < 0) {
-    m = m / (1.0 - (double)o.sumT / kP24);
-  } else {
-    m = m * o.A / ((double)o.T / kP24);
-    if (o.hit < NS) al = o.hit;
-    else be = o.hit - NS;
+      for (int b = 0; b < NS; ++b) Uc[a][b] = w.U[(int64_t)(a * NS + b) * nt + i];
+    decompose_ref_f64<NS>(M, w.R + i, nt, n, Uc, e0, U0);
+  }
+  unsigned int n_deg = 0, n_bad = 0;
+#pragma unroll 1
+  for (int32_t t = 0; t < len; ++t) {
+    double e1[NS], U1[NS][NS];
+    const StepN o = walker_stepN_f64<NS>(M, w.R + i, w.P + i, nt, n, al, be, phi, e0, U0, e1, U1,
+                                         dt, seed, traj_off + (uint64_t)i, step + t);
+    if (o.hit < 0) {
+      m = m / (1.0 - (double)o.sumT / kP24);
+    } else {
+      m = m * o.A / ((double)o.T / kP24);
+      if (o.hit < NS) al = o.hit;
+      else be = o.hit - NS;
+    }
+#pragma unroll
+    for (int a = 0; a < NS; ++a) {
+      e0[a] = e1[a];
+#pragma unroll
+      for (int b = 0; b < NS; ++b) U0[a][b] = U1[a][b];
+    }
+    n_deg += o.deg ? 1u : 0u;
+    n_bad += (!isfinite(m) || !isfinite(phi)) ? 1u : 0u;
   }
   w.m[i] = m;
   w.phi[i] = phi;
@@ -274,13 +305,13 @@ __global__ void __launch_bounds__(128) k_stepN_f64(const DevModel* __restrict__ 
 #pragma unroll
   for (int a = 0; a < NS; ++a)
 #pragma unroll
-    for (int b = 0; b < NS; ++b) w.U[(int64_t)(a * NS + b) * nt + i] = U1[a][b];
-  if (o.deg) {
-    atomicAdd(&w.hdr->n_degenerate, 1ull);
+    for (int b = 0; b < NS; ++b) w.U[(int64_t)(a * NS + b) * nt + i] = U0[a][b];
+  if (n_deg) {
+    atomicAdd(&w.hdr->n_degenerate, (unsigned long long)n_deg);
     atomicOr(&w.hdr->flags, QCL_FLAG_DEGENERATE);
   }
-  if (!isfinite(m) || !isfinite(phi)) {
-    atomicAdd(&w.hdr->n_nonfinite, 1ull);
+  if (n_bad) {
+    atomicAdd(&w.hdr->n_nonfinite, (unsigned long long)n_bad);
     atomicOr(&w.hdr->flags, QCL_FLAG_NONFINITE);
   }
 }
@@ -321,13 +352,13 @@ __device__ __forceinline__ double diag_pick(const double (&W)[NS][NS], int a) {
 
 // Diabatic pairs: the deterministic part and the draw (A = c, the real factor
 // of the event's amplitude; slot < NS takes three quarter turns, the others one).
+// W0 = W(R_n); W1 receives W(R_{n+1}).
 template <int NS>
 __device__ __forceinline__ StepN walker_stepN_dia_f64(const DevModel* __restrict__ M, double* R,
                                                       double* P, int64_t nt, int n, int al, int be,
-                                                      double& phi, double dt, uint64_t seed,
-                                                      uint64_t traj, int64_t step) {
-  double W0[NS][NS], W1[NS][NS];
-  elec_g<NS>(M, R, nt, n, W0);
+                                                      double& phi, const double (&W0)[NS][NS],
+                                                      double (&W1)[NS][NS], double dt,
+                                                      uint64_t seed, uint64_t traj, int64_t step) {
   dia_kick_g<NS>(M, R, P, nt, n, al, be, dt);
   for (int j = 0; j < n; ++j) R[(int64_t)j * nt] += dt * P[(int64_t)j * nt] / M->mass[j];
   elec_g<NS>(M, R, nt, n, W1);
@@ -373,11 +404,12 @@ __device__ __forceinline__ StepN walker_stepN_dia_f64(const DevModel* __restrict
   return draw_event<NC>(c, T, sumT, false, seed, traj, step);
 }
 
+// `len` steps of one walker per thread, W carried from step to step.
 template <int NS>
-__global__ void __launch_bounds__(128) k_stepN_dia_f64(const DevModel* __restrict__ M, void* buf,
+__global__ void __launch_bounds__(32) k_stepsN_dia_f64(const DevModel* __restrict__ M, void* buf,
                                                        int64_t nt, int n, int64_t step0,
-                                                       int64_t step, double dt, uint64_t seed,
-                                                       uint64_t traj_off) {
+                                                       int64_t step, int32_t len, double dt,
+                                                       uint64_t seed, uint64_t traj_off) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   WN<double> w = viewN<double>(buf, nt, NS, n, QCL_PREC_FP64);
   if (i >= nt) return;
@@ -388,25 +420,37 @@ __global__ void __launch_bounds__(128) k_stepN_dia_f64(const DevModel* __restric
   const uint16_t ab = w.ab[i];
   int al = ab & 0xf, be = (ab >> 8) & 0xf, q = (ab >> 4) & 3;
   double m = w.m[i], phi = w.phi[i];
-  const StepN o = walker_stepN_dia_f64<NS>(M, w.R + i, w.P + i, nt, n, al, be, phi, dt, seed,
-                                           traj_off + (uint64_t)i, step);
-  if (o.hit < 0) {
-    m = m / (1.0 - (double)o.sumT / kP24);
-  } else {
-    m = m * o.A / ((double)o.T / kP24);
-    if (o.hit < NS) {
-      al = o.hit;
-      q = (q + 3) & 3;
+  double W0[NS][NS];
+  elec_g<NS>(M, w.R + i, nt, n, W0);
+  unsigned int n_bad = 0;
+#pragma unroll 1
+  for (int32_t t = 0; t < len; ++t) {
+    double W1[NS][NS];
+    const StepN o = walker_stepN_dia_f64<NS>(M, w.R + i, w.P + i, nt, n, al, be, phi, W0, W1, dt,
+                                             seed, traj_off + (uint64_t)i, step + t);
+    if (o.hit < 0) {
+      m = m / (1.0 - (double)o.sumT / kP24);
     } else {
-      be = o.hit - NS;
-      q = (q + 1) & 3;
+      m = m * o.A / ((double)o.T / kP24);
+      if (o.hit < NS) {
+        al = o.hit;
+        q = (q + 3) & 3;
+      } else {
+        be = o.hit - NS;
+        q = (q + 1) & 3;
+      }
     }
+#pragma unroll
+    for (int a = 0; a < NS; ++a)
+#pragma unroll
+      for (int b = 0; b < NS; ++b) W0[a][b] = W1[a][b];
+    n_bad += (!isfinite(m) || !isfinite(phi)) ? 1u : 0u;
   }
   w.m[i] = m;
   w.phi[i] = phi;
   w.ab[i] = (uint16_t)(al | (q << 4) | (be << 8));
-  if (!isfinite(m) || !isfinite(phi)) {
-    atomicAdd(&w.hdr->n_nonfinite, 1ull);
+  if (n_bad) {
+    atomicAdd(&w.hdr->n_nonfinite, (unsigned long long)n_bad);
     atomicOr(&w.hdr->flags, QCL_FLAG_NONFINITE);
   }
 }
@@ -638,16 +682,19 @@ __global__ void __launch_bounds__(256) k_spawnN_step(const DevModel* __restrict_
       const double m = w.m[i];
       StepN o;
       if (dia) {
-        o = walker_stepN_dia_f64<NS>(M, w.R + i, w.P + i, cap, n, al, be, phi, dt, seed, w.id[i],
-                                     step);
+        double W0[NS][NS], W1[NS][NS];
+        elec_g<NS>(M, w.R + i, cap, n, W0);
+        o = walker_stepN_dia_f64<NS>(M, w.R + i, w.P + i, cap, n, al, be, phi, W0, W1, dt, seed,
+                                     w.id[i], step);
       } else {
-        double Uc[NS][NS], U1[NS][NS];
+        double Uc[NS][NS], e0[NS], U0[NS][NS], e1[NS], U1[NS][NS];
 #pragma unroll
         for (int a = 0; a < NS; ++a)
 #pragma unroll
           for (int b = 0; b < NS; ++b) Uc[a][b] = w.U[(int64_t)(a * NS + b) * cap + i];
-        o = walker_stepN_f64<NS>(M, w.R + i, w.P + i, cap, n, al, be, phi, Uc, U1, dt, seed,
-                                 w.id[i], step);
+        decompose_ref_f64<NS>(M, w.R + i, cap, n, Uc, e0, U0);
+        o = walker_stepN_f64<NS>(M, w.R + i, w.P + i, cap, n, al, be, phi, e0, U0, e1, U1, dt,
+                                 seed, w.id[i], step);
 #pragma unroll
         for (int a = 0; a < NS; ++a)
 #pragma unroll

@@ -24,12 +24,13 @@ struct NStateOps {
     k_sampleN_f32<NS><<<(unsigned)(nb > 0 ? nb : 1), 128, 0, st>>>(sp, buf);
   }
   static void step64(const DevModel* dm, int repr, void* buf, int64_t nt, int n, int64_t step0,
-                     int64_t step, double dt, uint64_t seed, uint64_t traj_off, cudaStream_t st) {
-    const unsigned nb = (unsigned)((nt + 127) / 128);
+                     int64_t step, int32_t len, double dt, uint64_t seed, uint64_t traj_off,
+                     cudaStream_t st) {
+    const unsigned nb = (unsigned)((nt + 31) / 32);
     if (repr == QCL_REPR_DIABATIC)
-      k_stepN_dia_f64<NS><<<nb, 128, 0, st>>>(dm, buf, nt, n, step0, step, dt, seed, traj_off);
+      k_stepsN_dia_f64<NS><<<nb, 32, 0, st>>>(dm, buf, nt, n, step0, step, len, dt, seed, traj_off);
     else
-      k_stepN_f64<NS><<<nb, 128, 0, st>>>(dm, buf, nt, n, step0, step, dt, seed, traj_off);
+      k_stepsN_f64<NS><<<nb, 32, 0, st>>>(dm, buf, nt, n, step0, step, len, dt, seed, traj_off);
   }
   static void observe64(const DevModel* dm, const void* buf, int64_t nt, int n, double* part,
                         cudaStream_t st) {

@@ -501,18 +501,31 @@ qcl_status qcl_propagate(const qcl_model* model, const qcl_ensemble_desc* ens, v
         first = false;
       }
     } else {
+      // output times wait in part's slots and are folded together
+      int slots = 0;
+      int64_t k_slot = 0;
+      auto flush = [&]() {
+        if (slots > 0) launch_fold(part, rows + (size_t)k_slot * q2, fold, OL.n_tiles, q2, slots, s, chunk_row(k_slot));
+        slots = 0;
+      };
       auto observe = [&](int64_t k) {
-        launch_observeN_f64(model->dev, ns, ens_buf, nt, model->n, part, s);
-        launch_fold(part, rows + (size_t)k * q2, fold, OL.n_tiles, q2, 1, s, chunk_row(k));
+        if (slots == 0) k_slot = k;
+        launch_observeN_f64(model->dev, ns, ens_buf, nt, model->n, part + (size_t)slots * OL.n_tiles * q2, s);
+        if (++slots == kChunkOut) flush();
       };
       if (step0 == 0) observe(0);
-      for (int64_t t = step0; t < end; ++t) {
+      for (int64_t t = step0; t < end;) {
+        // up to the next output time, at most 16 steps (a launch of 1e6 walkers then
+        // stays below a second)
+        const int64_t len = std::min<int64_t>(std::min<int64_t>(end, (t / out_stride + 1) * out_stride) - t, 16);
         {
           TimedLaunch tl(1, s);
-          launch_stepN_f64(model->dev, model->host.repr, ns, ens_buf, nt, model->n, step0, t, dt, ens->seed, ens->traj_id_offset, s);
+          launch_stepsN_f64(model->dev, model->host.repr, ns, ens_buf, nt, model->n, step0, t, (int32_t)len, dt, ens->seed, ens->traj_id_offset, s);
         }
-        if ((t + 1) % out_stride == 0) observe((t + 1) / out_stride);
+        t += len;
+        if (t % out_stride == 0) observe(t / out_stride);
       }
+      flush();
     }
     st = check_launch("FP64 step");
     if (st) return st;
