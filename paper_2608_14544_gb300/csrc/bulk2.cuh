@@ -350,11 +350,12 @@ __device__ __forceinline__ void sample_walker_f32(const Sample32& sp, uint64_t t
                                                   float* Pg, int64_t stride, float& mh,
                                                   uint16_t& ab) {
   const int n = sp.n;
+  const PhiloxStream rng(sp.seed, traj, kPurposeInit);
   float a = sp.a0, b = sp.b0;
   for (int j = 0; j < n; ++j) {
     float R = sp.R0[j], P = sp.P0[j];
     if (sp.wigner) {
-      const u4 wd = philox_draw(sp.seed, (uint32_t)j, traj, kPurposeInit);
+      const u4 wd = rng.draw((uint32_t)j);
       const float u0 = __fmaf_rn(__uint2float_rn(wd.x), 0x1p-32f, 0x1p-33f);
       const float u1 = __fmaf_rn(__uint2float_rn(wd.y), 0x1p-32f, 0x1p-33f);
       const float rad = sqrtf(-2.0f * logf(u0));
@@ -371,15 +372,13 @@ __device__ __forceinline__ void sample_walker_f32(const Sample32& sp, uint64_t t
   const float r2 = a * a + b * b;
   float c = 1.0f, s = 0.0f;
   if (r2 > 0.0f) {
+    // the larger of cos, sin theta and, from it, the smaller
     const float ir = rsqrtf(r2);
     const float c2 = a * ir, s2 = b * ir;
-    if (a >= 0.0f) {
-      c = sqrtf(0.5f + 0.5f * c2);
-      s = 0.5f * s2 / c;
-    } else {
-      s = copysignf(sqrtf(0.5f - 0.5f * c2), b);
-      c = 0.5f * s2 / s;
-    }
+    const float big = sqrtf(__fmaf_rn(0.5f, fabsf(c2), 0.5f));
+    const float small = 0.5f * fabsf(s2) / big;
+    c = a >= 0.0f ? big : small;
+    s = copysignf(a >= 0.0f ? small : big, b);
   }
   const float U[4] = {-s, c, c, s};
   float rho_ad[4];  // the density in the walkers' representation
@@ -412,7 +411,7 @@ __device__ __forceinline__ void sample_walker_f32(const Sample32& sp, uint64_t t
   }
   if (sumT <= 16777216u) Tk[last] += 16777216u - sumT;
   else Tk[big] -= sumT - 16777216u;
-  const u4 wd = philox_draw(sp.seed, (uint32_t)n, traj, kPurposeInit);
+  const u4 wd = rng.draw((uint32_t)n);
   const uint32_t y = wd.x >> 8;
   uint32_t cum = 0;
   int pick = last;

@@ -42,13 +42,17 @@ __device__ __forceinline__ void half_angle(const Ad2& d, double& c, double& s) {
     s = 0.0;
     return;
   }
-  if (d.a >= 0.0) {
-    c = sqrt((d.r + d.a) / (2.0 * d.r));
-    s = d.b / (2.0 * d.r * c);
-  } else {
-    s = copysign(sqrt((d.r - d.a) / (2.0 * d.r)), d.b);
-    c = d.b / (2.0 * d.r * s);
-  }
+  // the larger of cos, sin theta and, from it, the smaller
+  const double big = sqrt((d.r + fabs(d.a)) / (2.0 * d.r));
+  const double small = fabs(d.b) / (2.0 * d.r * big);
+  c = d.a >= 0.0 ? big : small;
+  s = copysign(d.a >= 0.0 ? small : big, d.b);
+}
+
+// (x + 1/2) 2^-32, exactly: the low bits of 2^19 + u, whose last place is 2^-33,
+// less 2^19 (one FP64 operation for a conversion, a sum and a product).
+__device__ __forceinline__ double uniform64(uint32_t x) {
+  return __dadd_rn(__hiloint2double((int)(0x41200000u | (x >> 31)), (int)(2u * x + 1u)), -0x1p19);
 }
 
 template <typename T>
@@ -96,8 +100,8 @@ __device__ __forceinline__ void sample_walker_f64(const DevModel* __restrict__ M
     double R = sp.R0[j], P = sp.P0[j];
     if (sp.wigner) {
       const u4 wd = philox_draw(sp.seed, (uint32_t)j, traj, kPurposeInit);
-      const double u0 = ((double)wd.x + 0.5) * 0x1p-32;
-      const double u1 = ((double)wd.y + 0.5) * 0x1p-32;
+      const double u0 = uniform64(wd.x);
+      const double u1 = uniform64(wd.y);
       const double rad = sqrt(-2.0 * log(u0));
       double sn, cs;
       sincospi(2.0 * u1, &sn, &cs);
@@ -123,8 +127,10 @@ __device__ __forceinline__ void sample_walker_f64(const DevModel* __restrict__ M
       if (M->repr == QCL_REPR_DIABATIC) {
         acc = sp.rho[al * 2 + be];
       } else {
+        // (zero elements of the density, most of a pure state's, add nothing)
         for (int k = 0; k < 2; ++k)
-          for (int l = 0; l < 2; ++l) acc += U[k * 2 + al] * sp.rho[k * 2 + l] * U[l * 2 + be];
+          for (int l = 0; l < 2; ++l)
+            if (sp.rho[k * 2 + l] != 0.0) acc += U[k * 2 + al] * sp.rho[k * 2 + l] * U[l * 2 + be];
       }
       rho_ad[al * 2 + be] = acc;
     }

@@ -57,8 +57,8 @@ inline void make_sample32(const DevModel& h, const SampleParams& sp, Sample32& s
 
 // The N_s-state FP32 sampler's inputs, converted to FP32 once on the host:
 // E (N_s x N_s), K_j (N_s x N_s each, j < n, when n N_s^2 <= kSampleNK; larger
-// models are read from the model's FP64 K on the device and rounded to FP32
-// there, the same values) and the initial density.
+// models are read from the model's FP32 copy of K on the device, the same values:
+// rounding the FP64 K there kept the FP64 unit 96 % busy) and the initial density.
 constexpr int kSampleNK = 512;
 struct SampleN32 {
   int64_t n_traj;
@@ -69,7 +69,7 @@ struct SampleN32 {
   float E[kMaxNS * kMaxNS];
   float rho[kMaxNS * kMaxNS];
   float K[kSampleNK];
-  const double* Kd;  // the model's K on the device, [n][N_s][N_s]
+  const float* Kd;  // the model's K in FP32 on the device, [n][N_s][N_s]
 };
 
 // FP32 per-mode coefficients of a two-state model for one time step dt.

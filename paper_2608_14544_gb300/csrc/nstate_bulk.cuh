@@ -39,15 +39,19 @@ __device__ __forceinline__ void sample_walkerN_f32(const SampleN32& sp, uint64_t
     }
     Rg[(int64_t)j * stride] = R;
     Pg[(int64_t)j * stride] = P;
-    const float* Kj = sp.K + j * NS * NS;
-    const double* Kdj = sp.Kd + (size_t)j * NS * NS;
+    if (k_dev) {
+      const float* Kj = sp.Kd + (size_t)j * NS * NS;
 #pragma unroll
-    for (int a = 0; a < NS; ++a)
+      for (int a = 0; a < NS; ++a)
 #pragma unroll
-      for (int b = 0; b < NS; ++b) {
-        const float kv = k_dev ? (float)Kdj[a * NS + b] : Kj[a * NS + b];
-        W[a][b] = __fmaf_rn(R, kv, W[a][b]);
-      }
+        for (int b = 0; b < NS; ++b) W[a][b] = __fmaf_rn(R, __ldg(Kj + a * NS + b), W[a][b]);
+    } else {
+      const float* Kj = sp.K + j * NS * NS;
+#pragma unroll
+      for (int a = 0; a < NS; ++a)
+#pragma unroll
+        for (int b = 0; b < NS; ++b) W[a][b] = __fmaf_rn(R, Kj[a * NS + b], W[a][b]);
+    }
   }
   eigh_ns<float, NS>(W, nullptr, e, U, 12, 1e-13f);
   // the pair's density: U^T rho U in the adiabatic basis, rho itself in the
@@ -478,13 +482,20 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
       // (a pointer for each array and a counter for the coefficients: the counter
       // stays warp-uniform)
       const char *Rj = Rt, *Pj = Pt;
-      float *rs = Rs, *ps = Ps;
+      uint32_t so = 0;
+      auto adv = [&](uint32_t by) {  // (opaque: not merged with the counter)
+        if (SM > 0) asm volatile("add.u32 %0, %0, %1;" : "+r"(so) : "r"(by));
+      };
+      auto at = [&](float* b) { return reinterpret_cast<float*>(reinterpret_cast<char*>(b) + so); };
       int j = 0;
-      for (; j + MU <= bp.n;
-           j += MU, Rj += MU * ms, Pj += MU * ms, rs += MU * TW, ps += MU * TW)
-        batch(j, std::integral_constant<int, MU>{}, Rj, Pj, rs, ps);
-      for (; j < bp.n; ++j, Rj += ms, Pj += ms, rs += TW, ps += TW)
-        batch(j, std::integral_constant<int, 1>{}, Rj, Pj, rs, ps);
+      for (; j + MU <= bp.n; j += MU, Rj += MU * ms, Pj += MU * ms) {
+        batch(j, std::integral_constant<int, MU>{}, Rj, Pj, at(Rs), at(Ps));
+        adv(4u * MU * TW);
+      }
+      for (; j < bp.n; ++j, Rj += ms, Pj += ms) {
+        batch(j, std::integral_constant<int, 1>{}, Rj, Pj, at(Rs), at(Ps));
+        adv(4u * TW);
+      }
     };
     auto pass_a = [&](const V (&Q)[NTRI], V (&W)[NS][NS]) {
       V t[NTRI];

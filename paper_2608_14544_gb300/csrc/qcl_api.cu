@@ -276,15 +276,18 @@ qcl_status qcl_create_model(const qcl_model_desc* d, qcl_model** out) {
   cudaGetDevice(&dev);
   m->device = dev;
   char* blk = nullptr;
-  const size_t bytes = sizeof(DevModel) + sizeof(double) * nn * n;
+  const size_t bytes = sizeof(DevModel) + (sizeof(double) + sizeof(float)) * nn * n;
   cudaError_t e = cudaMalloc((void**)&blk, bytes);
   if (e != cudaSuccess) {
     delete m;
     return fail(e == cudaErrorMemoryAllocation ? QCL_ERR_OUT_OF_MEMORY : QCL_ERR_CUDA, "cudaMalloc of the model block failed: %s", cudaGetErrorString(e));
   }
   h.K = (const double*)(blk + sizeof(DevModel));
+  h.K32 = (const float*)(blk + sizeof(DevModel) + sizeof(double) * nn * n);
+  const std::vector<float> k32(m->K.begin(), m->K.end());
   e = cudaMemcpy(blk, &h, sizeof(DevModel), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(blk + sizeof(DevModel), d->K, sizeof(double) * nn * n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy((void*)h.K32, k32.data(), sizeof(float) * nn * n, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(blk);
     delete m;
@@ -380,7 +383,7 @@ void make_sampleN32(const qcl_model* model, const SampleParams& sp, SampleN32& s
   }
   const size_t nk = (size_t)n * ns * ns;
   for (size_t k = 0; k < (size_t)kSampleNK; ++k) s.K[k] = k < nk ? (float)model->K[k] : 0.0f;
-  s.Kd = model->host.K;
+  s.Kd = model->host.K32;
 }
 
 // Validates an initial condition and builds the sampling parameters.

@@ -172,8 +172,9 @@ struct DevModel {
   double mass[kMaxN], omega[kMaxN], k[kMaxN];
   double a[kMaxN], b[kMaxN], s[kMaxN];
   double E[kMaxNS * kMaxNS];
-  // K[j][ns*ns] follows in a separate allocation (pointer below)
+  // K[j][ns*ns] and its FP32 rounding follow in the same allocation
   const double* K;
+  const float* K32;
 };
 
 // ------------------------------------------------------------------ layouts --
