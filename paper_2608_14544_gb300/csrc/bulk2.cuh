@@ -133,12 +133,14 @@ __device__ __forceinline__ void set_lane(Scal& z, int, const Scal& o) { z = o; }
 // is undefined and the coupling is set to zero) both come out 0 -- the mean of
 // the two branches -- instead of a division by zero.
 // S2 = false leaves s2 stale (the spin-boson step needs no sin 2theta; the
-// observation recomputes it).
-template <bool S2 = true, typename V>
+// observation recomputes it).  FLOOR = false leaves out the floor (the spin-boson
+// form, whose r^2 >= b0^2 lies above it).
+template <bool S2 = true, bool FLOOR = true, typename V>
 __device__ __forceinline__ void closed_form(ScalV<V>& z) {
   z.r2 = vfma(z.A, z.A, vmul(z.B, z.B));
 #pragma unroll
-  for (int l = 0; l < Lanes<V>::W; ++l) ln(z.ir, l) = rsqrt_normal(fmaxf(ln(z.r2, l), 0x1p-126f));
+  for (int l = 0; l < Lanes<V>::W; ++l)
+    ln(z.ir, l) = rsqrt_normal(FLOOR ? fmaxf(ln(z.r2, l), 0x1p-126f) : ln(z.r2, l));
   z.r = vmul(z.r2, z.ir);
   z.c2 = vmul(z.A, z.ir);
   if (S2) z.s2 = vmul(z.B, z.ir);
@@ -817,7 +819,7 @@ __device__ __forceinline__ void bulk2_tile(const BulkParams& bp, const CF& cf, W
       z.A = vfma(splat<V>(cf.a[j]), w.R[j], z.A);
       if (KIND == 1) z.B = vfma(splat<V>(cf.b[j]), w.R[j], z.B);
     }
-    closed_form<KIND == 1>(z);
+    closed_form<KIND == 1, KIND == 1>(z);
     kick<NPL, KIND, CF>(w, cf, vmul(hsab, z.c2), vmul(hsab, z.s2));  // second half kick at R_{n+1}
     V Av = splat<V>(0.0f), Bv = splat<V>(0.0f);
 #pragma unroll

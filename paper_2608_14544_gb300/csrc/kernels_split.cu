@@ -249,7 +249,7 @@ __device__ __forceinline__ void split_tiles_v(const BulkParams& bp, const Coef2&
       xsel ^= 1;
       z.A = vadd(splat<V>(bp.a0), v.v[0]);
       z.B = vadd(splat<V>(bp.b0), (KIND == 1) ? v.v[2] : splat<V>(0.0f));
-      closed_form<KIND == 1>(z);
+      closed_form<KIND == 1, KIND == 1>(z);
       const V hu2 = vmul(hsab, z.c2), hv2 = vmul(hsab, z.s2);
 #pragma unroll
       for (int t = 0; t < NPL; ++t) {  // coupling terms of the second half kick at R_{n+1}
