@@ -275,19 +275,25 @@ qcl_status qcl_create_model(const qcl_model_desc* d, qcl_model** out) {
   int dev = 0;
   cudaGetDevice(&dev);
   m->device = dev;
+  // one block, one copy: the model, K and K rounded to FP32
   char* blk = nullptr;
-  const size_t bytes = sizeof(DevModel) + (sizeof(double) + sizeof(float)) * nn * n;
+  const size_t off_k = sizeof(DevModel), off_k32 = off_k + sizeof(double) * nn * n;
+  const size_t bytes = off_k32 + sizeof(float) * nn * n;
+  std::vector<char> image(bytes);
   cudaError_t e = cudaMalloc((void**)&blk, bytes);
   if (e != cudaSuccess) {
     delete m;
     return fail(e == cudaErrorMemoryAllocation ? QCL_ERR_OUT_OF_MEMORY : QCL_ERR_CUDA, "cudaMalloc of the model block failed: %s", cudaGetErrorString(e));
   }
-  h.K = (const double*)(blk + sizeof(DevModel));
-  h.K32 = (const float*)(blk + sizeof(DevModel) + sizeof(double) * nn * n);
-  const std::vector<float> k32(m->K.begin(), m->K.end());
-  e = cudaMemcpy(blk, &h, sizeof(DevModel), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(blk + sizeof(DevModel), d->K, sizeof(double) * nn * n, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy((void*)h.K32, k32.data(), sizeof(float) * nn * n, cudaMemcpyHostToDevice);
+  h.K = (const double*)(blk + off_k);
+  h.K32 = (const float*)(blk + off_k32);
+  memcpy(image.data(), &h, sizeof(DevModel));
+  memcpy(image.data() + off_k, d->K, sizeof(double) * nn * n);
+  for (size_t k = 0; k < nn * n; ++k) {
+    const float x = (float)d->K[k];
+    memcpy(image.data() + off_k32 + k * sizeof(float), &x, sizeof(float));
+  }
+  e = cudaMemcpy(blk, image.data(), bytes, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(blk);
     delete m;
