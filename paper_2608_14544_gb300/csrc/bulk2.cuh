@@ -428,44 +428,53 @@ __device__ __forceinline__ void sample_walker_f32(const Sample32& sp, uint64_t t
   ab = (uint16_t)((pick >> 1) | ((pick & 1) << 8));
 }
 
-// Transition test of a spawning walker (the scheme that starts a new walker
-// whenever the test fires): the phase as in phase_and_transition (DIA: as in
-// dia_phase_and_transition, w_old = a(R_n), Bv = b(R_{n+1})); when the test
-// fires for event e, `child` becomes a copy of the walker with its weight times
-// A_e / p_hat_e, the flipped index and (DIA) the event's quarter turns, and the
-// walker keeps its pair and weight (no stay factor).  Returns whether it fired.
+// Threshold T (of 2^24, one event's share) and A_e 2^24 of the first-index event
+// (fac; DIA: of both events) of a spawning walker's test, from its state at
+// R_{n+1}.  Returns whether the gap is degenerate.
 template <int KIND, bool DIA>
-__device__ __forceinline__ bool spawn_transition(Scal& z, float w_old, float Av, float Bv,
-                                                 uint32_t word, const BulkParams& bp,
-                                                 unsigned int& deg, Scal& child) {
-  uint32_t T;
-  float fac;  // A_e 2^24 of the first-index event (DIA: both events)
+__device__ __forceinline__ bool spawn_rate(const Scal& z, float Av, float Bv, const BulkParams& bp,
+                                           uint32_t& T, float& fac) {
   if (DIA) {
-    z.ph.lo = __fmaf_rn(bp.hdt_hbar * (z.sb - z.sa), w_old + z.A, z.ph.lo);
     T = min(__float2uint_rz((bp.kamp * kP24f) * fabsf(Bv)), bp.tmax >> 1);
     fac = (bp.amp * kP24f) * Bv;
-  } else {
-    z.ph.lo = __fmaf_rn(bp.hdt_hbar * (z.sa - z.sb), w_old + z.r, z.ph.lo);
-    const bool degen = z.r2 < kDegR2_32;
-    deg += degen ? 1u : 0u;
-    const float gn = (KIND == 1) ? 0.5f * (z.A * Bv - z.B * Av) : (-0.5f * bp.b0) * Av;
-    const float g = degen ? 0.0f : gn * (z.ir * z.ir);
-    T = min(__float2uint_rz((bp.kamp * kP24f) * fabsf(g)), bp.tmax >> 1);
-    fac = (bp.amp * kP24f) * g;
+    return false;
   }
+  const bool degen = z.r2 < kDegR2_32;
+  const float gn = (KIND == 1) ? 0.5f * (z.A * Bv - z.B * Av) : (-0.5f * bp.b0) * Av;
+  const float g = degen ? 0.0f : gn * (z.ir * z.ir);
+  T = min(__float2uint_rz((bp.kamp * kP24f) * fabsf(g)), bp.tmax >> 1);
+  fac = (bp.amp * kP24f) * g;
+  return degen;
+}
+
+// Transition test of a spawning walker (the scheme that starts a new walker
+// whenever the test fires): the phase as in phase_and_transition (DIA: as in
+// dia_phase_and_transition, w_old = a(R_n), Bv = b(R_{n+1})), and the event that
+// fires: 0 none, 1 the first index, 2 the second.
+template <int KIND, bool DIA>
+__device__ __forceinline__ int spawn_event(Scal& z, float w_old, float Av, float Bv, uint32_t word,
+                                           const BulkParams& bp, unsigned int& deg, uint32_t& T,
+                                           float& fac) {
+  if (DIA) z.ph.lo = __fmaf_rn(bp.hdt_hbar * (z.sb - z.sa), w_old + z.A, z.ph.lo);
+  else z.ph.lo = __fmaf_rn(bp.hdt_hbar * (z.sa - z.sb), w_old + z.r, z.ph.lo);
+  deg += spawn_rate<KIND, DIA>(z, Av, Bv, bp, T, fac) ? 1u : 0u;
   const uint32_t y = word >> 8;
-  const bool hop1 = y < T;
-  const bool hop = y < 2u * T;
-  if (!hop) return false;
-  child = z;
+  return y < T ? 1 : (y < 2u * T ? 2 : 0);
+}
+
+// Makes `child`, a copy of the walker whose test fired for event `ev`, the new
+// walker: its weight times A_e / p_hat_e, the flipped index and (DIA) the event's
+// quarter turns.  (The walker keeps its pair and weight: no stay factor.)
+template <bool DIA>
+__device__ __forceinline__ void spawn_child(Scal& child, int ev, uint32_t T, float fac) {
+  const bool hop1 = ev == 1;
   // adiabatic: A_1 = -sig_a dt g, A_2 = -sig_b dt g; diabatic: both c = b dt / hbar
-  const float num = DIA ? fac : -(hop1 ? z.sa : z.sb) * fac;
+  const float num = DIA ? fac : -(hop1 ? child.sa : child.sb) * fac;
   weight_factor(child, num, __uint2float_rn(T));
   child.m = fast_two_sum(child.m.hi, child.m.lo);
   if (hop1) child.sa = -child.sa;
   else child.sb = -child.sb;
   if (DIA) child.q = (child.q + (hop1 ? 3 : 1)) & 3;
-  return true;
 }
 
 // Keeps the stored phase within about 2^10 rad, where the three-part

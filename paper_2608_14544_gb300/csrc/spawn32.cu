@@ -94,10 +94,8 @@ __device__ __forceinline__ void spawn_phase_end(Scal& z, int64_t step) {
   }
 }
 
-// What a step reports: a non-finite child or phase, a degenerate gap.
-__device__ __forceinline__ void spawn_report(EnsHeader* hdr, const Scal& z, bool hop,
-                                             const Scal& child, unsigned int deg) {
-  const unsigned bad = (hop && !isfinite(child.m.hi) ? 1u : 0u) + (!isfinite(z.ph.hi) ? 1u : 0u);
+// What a step reports: non-finite children or phases, a degenerate gap.
+__device__ __forceinline__ void spawn_report(EnsHeader* hdr, unsigned int bad, unsigned int deg) {
   if (bad) {
     atomicAdd(&hdr->n_nonfinite, (unsigned long long)bad);
     atomicOr(&hdr->flags, QCL_FLAG_NONFINITE);
@@ -136,17 +134,10 @@ __device__ __forceinline__ void put_walker(const Set32& s, int64_t cap, int n, i
   s.fam[pos] = fam;
 }
 
-// One step of the walker x (random stream id) in registers: x moves to the next
-// step (its weight and pair stay), and where its test fires the result is true
-// and cm, cme, cab are the child's weight and pair.  REPORT counts degenerate
-// gaps and non-finite values in the header.
+// The weight, phase and pair of x as the step's scalars, and a and b at its R.
 template <int NPL, int KIND, bool DIA>
-__device__ __forceinline__ bool step_walker(const BulkParams& bp, const CoefLocal<NPL>& cf,
-                                            EnsHeader* hdr, int64_t step, SWalker<NPL>& x,
-                                            uint64_t id, f2& cm, int32_t& cme, uint16_t& cab,
-                                            bool report) {
-  using CF = CoefLocal<NPL>;
-  Walker<NPL>& w = x.w;
+__device__ __forceinline__ Scal walker_scal(const BulkParams& bp, const CoefLocal<NPL>& cf,
+                                            const SWalker<NPL>& x) {
   Scal z;
   z.m = x.m;
   z.mexp = x.me;
@@ -158,15 +149,41 @@ __device__ __forceinline__ bool step_walker(const BulkParams& bp, const CoefLoca
   z.B = bp.b0;
 #pragma unroll
   for (int j = 0; j < NPL; ++j) {
-    z.A = __fmaf_rn(cf.a[j], w.R[j], z.A);
-    if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
+    z.A = __fmaf_rn(cf.a[j], x.w.R[j], z.A);
+    if (KIND == 1) z.B = __fmaf_rn(cf.b[j], x.w.R[j], z.B);
   }
+  return z;
+}
+
+// The couplings' sums over P.
+template <int NPL, int KIND>
+__device__ __forceinline__ void coupling_sums(const CoefLocal<NPL>& cf, const Walker<NPL>& w,
+                                              float& Av, float& Bv) {
+  Av = Bv = 0.0f;
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) {
+    Av = __fmaf_rn(cf.am[j], w.P[j], Av);
+    if (KIND == 1) Bv = __fmaf_rn(cf.bm[j], w.P[j], Bv);
+  }
+}
+
+// One step of the walker x (random stream id) in registers: x moves to the next
+// step (its weight and pair stay); returns the event its test fires for (0 none).
+// `report` counts degenerate gaps and non-finite phases in the header.
+template <int NPL, int KIND, bool DIA>
+__device__ __forceinline__ int step_walker(const BulkParams& bp, const CoefLocal<NPL>& cf,
+                                           EnsHeader* hdr, int64_t step, SWalker<NPL>& x,
+                                           uint64_t id, bool report) {
+  using CF = CoefLocal<NPL>;
+  Walker<NPL>& w = x.w;
+  Scal z = walker_scal<NPL, KIND, DIA>(bp, cf, x);
   closed_form(z);
   const u4 wd = philox_draw(bp.seed, (uint32_t)(step >> 2), id, kPurposeHop);
   const uint32_t word = word_of(wd, (int)(step & 3));
   unsigned int deg = 0;
-  Scal child;
-  bool hop;
+  uint32_t T;
+  float fac;
+  int ev;
   const float hsab = bp.hdt * 0.5f * (z.sa + z.sb);
   if (DIA) {
     kick_dia<NPL, KIND, CF>(w, cf, hsab);
@@ -181,7 +198,7 @@ __device__ __forceinline__ bool step_walker(const BulkParams& bp, const CoefLoca
       if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
     }
     kick_dia<NPL, KIND, CF>(w, cf, hsab);
-    hop = spawn_transition<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, child);
+    ev = spawn_event<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, T, fac);
   } else {
     kick<NPL, KIND, CF>(w, cf, hsab * z.c2, hsab * z.s2);
 #pragma unroll
@@ -196,24 +213,38 @@ __device__ __forceinline__ bool step_walker(const BulkParams& bp, const CoefLoca
     }
     closed_form(z);
     kick<NPL, KIND, CF>(w, cf, hsab * z.c2, hsab * z.s2);
-    float Av = 0.0f, Bv = 0.0f;
-#pragma unroll
-    for (int j = 0; j < NPL; ++j) {
-      Av = __fmaf_rn(cf.am[j], w.P[j], Av);
-      if (KIND == 1) Bv = __fmaf_rn(cf.bm[j], w.P[j], Bv);
-    }
-    hop = spawn_transition<KIND, false>(z, r_old, Av, Bv, word, bp, deg, child);
+    float Av, Bv;
+    coupling_sums<NPL, KIND>(cf, w, Av, Bv);
+    ev = spawn_event<KIND, false>(z, r_old, Av, Bv, word, bp, deg, T, fac);
   }
   spawn_phase_end(z, step);
   x.ph = z.ph;
-  if (hop) {
-    renorm(child.m, child.mexp);
-    cm = child.m;
-    cme = child.mexp;
-    cab = pair_word(child);
+  if (report) spawn_report(hdr, !isfinite(z.ph.hi) ? 1u : 0u, deg);
+  return ev;
+}
+
+// The child of the walker x whose step has fired for event ev, from x after that
+// step: the test's threshold follows from R and P again.  Returns false when its
+// weight is not finite.
+template <int NPL, int KIND, bool DIA>
+__device__ __forceinline__ bool make_child(const BulkParams& bp, const CoefLocal<NPL>& cf,
+                                           const SWalker<NPL>& x, int ev, SWalker<NPL>& c) {
+  Scal z = walker_scal<NPL, KIND, DIA>(bp, cf, x);
+  float Av = 0.0f, Bv = z.B;
+  if (!DIA) {
+    closed_form(z);
+    coupling_sums<NPL, KIND>(cf, x.w, Av, Bv);
   }
-  if (report) spawn_report(hdr, z, hop, child, deg);
-  return hop;
+  uint32_t T;
+  float fac;
+  spawn_rate<KIND, DIA>(z, Av, Bv, bp, T, fac);
+  spawn_child<DIA>(z, ev, T, fac);
+  renorm(z.m, z.mexp);
+  c = x;
+  c.m = z.m;
+  c.me = z.mexp;
+  c.ab = pair_word(z);
+  return isfinite(z.m.hi);
 }
 
 // The chained steps' counts: children of each 256-walker group of the current
@@ -244,23 +275,30 @@ __device__ __forceinline__ void add_counts(unsigned int* cnt, bool fires, int64_
 // evaluated, beside its own step, which of its walkers fire at the next one, and
 // counted them by the group of 256 positions they stand in.  So a block learns
 // the children before its walkers by adding the counts of the groups before
-// them, steps its walkers in registers, writes each with its child straight to
-// its place, and evaluates the step after for the counts of the next launch
-// (FIRST only counts, for a call's first step).  Nothing waits inside a launch,
-// and an overflow is known at its start: then the step's children are dropped.
+// them, writes each walker with its child straight to its place, and evaluates
+// the step after for the counts of the next launch (FIRST only counts, for a
+// call's first step).  Nothing waits inside a launch, and an overflow is known at
+// its start: then the step's children are dropped.
 //
-// What bounds it: instruction issue at 1e6 walkers (698 instructions a warp of
-// walkers, of which the two evaluations of the step are 360; 40 us a step against
-// 15 us for its bytes), launch latency below some 1e5 (8-12 us a step).  1e5
-// initial one-mode walkers growing to 1.55e6 over 400 steps: 10.0 ms of device
-// time, where a step in place, a one-block scan and a scatter took 15.9 ms.  One
-// cooperative launch for many steps, with a decoupled look-back over the groups'
-// counts and a grid barrier, was slower (13.6 ms): a poll of another die's word
-// costs about a microsecond, and a step needs several in a row.
+// `out`: the walkers are written as the step after leaves them, with the event
+// that fired (0, 1, 2) in the top two bits of the pair word, and the next launch
+// (`in`) has only to place them and to make the children of the few that fired.
+// So a step is evaluated once; at the ends of an interval between output times,
+// where the set has to hold the plain state, the step is evaluated for its counts
+// and again by the next launch.
+//
+// What bounds it: instruction issue at 1e6 walkers, launch latency below some 1e5
+// (7 us a step).  1e5 initial one-mode walkers growing to 1.57e6 over 400 steps
+// with an output every 10: 7.0 ms of device time; 10.0 ms when every launch
+// evaluated its own step again, 15.9 ms with a step in place, a one-block scan
+// and a scatter.  One cooperative launch for many steps, with a decoupled
+// look-back over the groups' counts and a grid barrier, was slower (13.6 ms): a
+// poll of another die's word costs about a microsecond, and a step needs several
+// in a row.
 template <int NPL, int KIND, bool DIA, bool FIRST>
 __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
     k_spawn_chain32(const BulkParams bp, const CoefLocal<NPL> cf, const SpawnLayout L, void* buf,
-                    int64_t cap, int64_t step) {
+                    int64_t cap, int64_t step, int in, int out) {
   __shared__ int wcnt[2][8];
   __shared__ unsigned long long wsum[8];
   EnsHeader* hdr = (EnsHeader*)buf;
@@ -287,6 +325,7 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
   SWalker<NPL> x;
   uint64_t id = 0;
   uint32_t fam = 0;
+  int ev = 0;  // the event x's step fired for
   auto load = [&](int64_t g) {
     const int64_t i = g * 256 + threadIdx.x;
     const int64_t ii = i < n_live ? i : 0;
@@ -299,7 +338,9 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
     x.m = {s.mh[ii], s.ml[ii]};
     x.me = s.me[ii];
     x.ph = {s.ph[ii], s.pl[ii]};
-    x.ab = s.ab[ii];
+    const unsigned ab = s.ab[ii];
+    x.ab = (uint16_t)(ab & 0x3fffu);
+    ev = (int)(ab >> 14);
     id = s.id[ii];
     fam = s.fam[ii];
   };
@@ -330,27 +371,19 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
     const int64_t i = g * 256 + threadIdx.x;
     const bool live = i < n_live;
     if (g > g0) load(g);
-    // phase 0: the step itself; 1: the walkers' next step; 2: their children's.
-    // One copy of the step's code, so that a walker's test comes out the same
-    // when it is counted and when it is taken.
+    // phase 0: the step itself, of walkers not moved yet; 1: the walkers' next
+    // step; 2: their children's.  One copy of the step's code, so that a walker's
+    // test comes out the same when it is only counted and when it is taken.
     SWalker<NPL> xc;      // the children
     uint64_t idc = 0;
     bool hop = false;
     int64_t pos = i;
 #pragma unroll 1
-    for (int phase = FIRST ? 1 : 0; phase < 3; ++phase) {
-      if (phase == 2) {
-        if (FIRST || !__any_sync(0xffffffffu, hop)) break;
-        x = xc;
-        id = idc;
-      }
-      f2 cm;
-      int32_t cme;
-      uint16_t cab;
-      const bool fires = step_walker<NPL, KIND, DIA>(bp, cf, hdr, FIRST || phase == 0 ? step : step + 1,
-                                                     x, id, cm, cme, cab, phase == 0 && live);
-      if (phase == 0) {
-        hop = fires && live && !drop;
+    for (int phase = FIRST || in ? 1 : 0; phase < 3; ++phase) {
+      if (!FIRST && phase == 1) {  // the walkers have moved: children and places
+        hop = ev != 0 && live;
+        if (hop && !make_child<NPL, KIND, DIA>(bp, cf, x, ev, xc)) spawn_report(hdr, 1u, 0u);
+        hop = hop && !drop;
         const unsigned bal = __ballot_sync(0xffffffffu, hop);
         int* const wc = wcnt[(g - g0) & 1];  // (two in turn: one barrier a group)
         if (lane == 0) wc[warp] = __popc(bal);
@@ -363,19 +396,30 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
         }
         pos = i + prefix + before;
         prefix += c;
-        if (live) put_walker(d, cap, bp.n, pos, x, id, fam);
-        if (hop) {
-          xc = x;
-          xc.m = cm;
-          xc.me = cme;
-          xc.ab = cab;
-          idc = child_id32(bp.seed, step, id);
-          put_walker(d, cap, bp.n, pos + 1, xc, idc, fam);
+        if (hop) idc = child_id32(bp.seed, step, id);
+        if (!out) {
+          if (live) put_walker(d, cap, bp.n, pos, x, id, fam);
+          if (hop) put_walker(d, cap, bp.n, pos + 1, xc, idc, fam);
         }
-      } else {
-        const bool f = fires && (phase == 1 ? live : hop);
-        add_counts(nxt, f, phase == 1 ? pos : pos + 1);
+      }
+      bool on = live;
+      if (phase == 2) {
+        if (FIRST || !__any_sync(0xffffffffu, hop)) break;
+        x = xc;
+        id = idc;
+        on = hop;
+        ++pos;
+      }
+      ev = step_walker<NPL, KIND, DIA>(bp, cf, hdr, FIRST || phase == 0 ? step : step + 1, x, id,
+                                       on && (phase == 0 || (!FIRST && out)));
+      if (phase > 0) {
+        const bool f = on && ev != 0;
+        add_counts(nxt, f, pos);
         found += __popc(__ballot_sync(0xffffffffu, f));
+        if (!FIRST && out && on) {
+          x.ab |= (uint16_t)(ev << 14);
+          put_walker(d, cap, bp.n, pos, x, id, fam);
+        }
       }
     }
   }
@@ -437,8 +481,9 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
       const u4 wd = philox_draw(bp.seed, (uint32_t)(step >> 2), s.id[i], kPurposeHop);
       const uint32_t word = word_of(wd, (int)(step & 3));
       unsigned int deg = 0;
-      Scal child;
-      bool hop;
+      uint32_t T;
+      float fac;
+      int ev;
       const float hsab = bp.hdt * 0.5f * (z.sa + z.sb);
       // P += dt/2 F with the pair's force (kick / kick_dia of one mode)
       auto kick1 = [&](int j, float r, float p, float hu, float hv) {
@@ -462,7 +507,7 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
           s.R[(int64_t)j * cap + i] = r;
           s.P[(int64_t)j * cap + i] = kick1(j, r, p, 0.0f, 0.0f);
         }
-        hop = spawn_transition<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, child);
+        ev = spawn_event<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, T, fac);
       } else {
         const float hu = hsab * z.c2, hv = hsab * z.s2;
         const float r_old = z.r;
@@ -487,8 +532,11 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
           if (KIND == 1) Bv = __fmaf_rn(cf.bm[j], p, Bv);
           s.P[(int64_t)j * cap + i] = p;
         }
-        hop = spawn_transition<KIND, false>(z, r_old, Av, Bv, word, bp, deg, child);
+        ev = spawn_event<KIND, false>(z, r_old, Av, Bv, word, bp, deg, T, fac);
       }
+      Scal child = z;
+      const bool hop = ev != 0;
+      if (hop) spawn_child<DIA>(child, ev, T, fac);
       spawn_phase_end(z, step);
       s.ph[i] = z.ph.hi;
       s.pl[i] = z.ph.lo;
@@ -502,7 +550,7 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
         ((int32_t*)((char*)buf + L.cmexp))[i] = child.mexp;
         ((uint16_t*)((char*)buf + L.cab))[i] = pair_word(child);
       }
-      spawn_report(hdr, z, hop, child, deg);
+      spawn_report(hdr, (hop && !isfinite(child.m.hi) ? 1u : 0u) + (!isfinite(z.ph.hi) ? 1u : 0u), deg);
     }
     const int cnt = __syncthreads_count(flag);
     if (threadIdx.x == 0) ((int32_t*)((char*)buf + L.bsum))[vb] = cnt;
@@ -716,20 +764,20 @@ void run_steps32(const BulkParams& bp, const Coef2& c2, void* buf, int64_t cap, 
   }
   const SpawnLayout L = SpawnLayout::make(cap, bp.n, n0, QCL_PREC_FP32_BULK);
   // every block resident at once (at most one group a block)
-  static int per_sm = 0;
-  if (per_sm == 0) {
+  static const int per_sm = [] {
     int b = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_spawn_chain32<NPL, KIND, DIA, false>, 256, 0);
-    per_sm = b < 1 ? 1 : b;
-  }
+    return b < 1 ? 1 : b;
+  }();
   const unsigned grid = spawn_grid(cap, per_sm);
   if (step == bp.step0) {
     k_spawn_chain_clear<<<grid, 256, 0, st>>>(buf, cap, bp.n, n0);
-    k_spawn_chain32<NPL, KIND, DIA, true><<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, step);
+    k_spawn_chain32<NPL, KIND, DIA, true><<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, step, 0, 0);
     launches_add(2);
   }
   for (int64_t t = step; t < step + len; ++t)
-    k_spawn_chain32<NPL, KIND, DIA, false><<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, t);
+    k_spawn_chain32<NPL, KIND, DIA, false>
+        <<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, t, t > step, t + 1 < step + len);
   launches_add(len);
 }
 

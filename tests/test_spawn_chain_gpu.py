@@ -65,3 +65,32 @@ def test_chained_steps_and_families(q, cfg_id, rep, n0, cap, kappa):
             # (each contribution rounds to FP32, phases by the fast sine: 2e-6 of |z|)
             assert abs(row[own + 2 * k + c] - X.sum()) <= 2e-6 * A.sum() + 1e-30
             assert abs(row[16 + own + 2 * k + c] - (X * X).sum()) <= 4e-6 * (A * A).sum() + 1e-30
+
+
+@pytest.mark.parametrize("rep", ["adiabatic", "diabatic"])
+@pytest.mark.parametrize("stride,splits", [(1, (4, 3)), (2, (4, 5)), (3, (2, 1, 7)), (50, (1, 6, 49))])
+def test_steps_between_outputs(q, rep, stride, splits):
+    """Intervals of one, two and more steps, cut by output times and by the
+    call's end: the same walkers and rows as the three-launch route."""
+    cfg = copy.deepcopy(wl.config(3))
+    cfg["model"]["repr"] = rep
+    cfg["model"]["hop_scale"] = 20.0
+    got = []
+    for mem in (0, 1):
+        q.set_option(q.OPT_MODES_IN_MEMORY, mem)
+        try:
+            r = q.SpawnRun(q.Model(cfg["model"]), 300, 60_000, 5, sum(splits) // stride + 1,
+                           precision=q.PREC_FP32_BULK)
+            r.sample(cfg["init"])
+            for n in splits:
+                r.propagate(n, cfg["dt"], stride)
+        finally:
+            q.set_option(q.OPT_MODES_IN_MEMORY, 0)
+        got.append(r)
+    a, b = got
+    assert a.n_live() == b.n_live() > 300
+    assert a.status() == b.status()
+    sa, sb = a.state(), b.state()
+    for key in sa:
+        assert np.array_equal(sa[key], sb[key]), key
+    assert np.array_equal(a.sums(), b.sums())
