@@ -980,8 +980,11 @@ qcl_status qcl_spawn_propagate(const qcl_model* model, const qcl_ensemble_desc* 
   if (k_last >= n_out) return fail(QCL_ERR_INVALID_ARG, "output row %lld beyond n_out = %lld", (long long)k_last, (long long)n_out);
   const SpawnLayout SL = SpawnLayout::make(capacity, model->n, ens->n_traj, ens->precision, model->ns);
   if (bytes < SL.total) return fail(QCL_ERR_OUT_OF_MEMORY, "buf has %zu bytes, needs %zu", bytes, SL.total);
-  // tiles of families as the ensemble's own tiles: 256 (two states, <= 32 modes in
-  // FP32), 128 for FP32 N_s-state models
+  // Tiles of families: 256, and 128 for FP32 N_s-state models.  (The buffer has
+  // room for the ensemble's own tiles, which hold fewer walkers for two states
+  // above 32 modes in FP32; the observation writes only the families' tiles.)
+  const int64_t n_tiles = ens->precision == QCL_PREC_FP32_BULK && model->ns > 2 ? (ens->n_traj + 127) / 128
+                                                                                : (ens->n_traj + 255) / 256;
   const ObsLayout OL = ObsLayout::make(ens->n_traj, model->ns, n_out, tile_walkers(ens->precision, model->n, model->ns));
   if (obs_bytes < OL.total) return fail(QCL_ERR_OUT_OF_MEMORY, "obs_buf has %zu bytes, needs %zu", obs_bytes, OL.total);
   cudaStream_t s = (cudaStream_t)stream;
@@ -1022,7 +1025,7 @@ qcl_status qcl_spawn_propagate(const qcl_model* model, const qcl_ensemble_desc* 
       launch_spawnN_observe(model->dev, model->ns, buf, capacity, model->n, n0, (int)(step & 1), part, s);
     else
       launch_spawn_observe(model->dev, buf, capacity, model->n, n0, (int)(step & 1), part, s);
-    launch_fold(part, row, fold, OL.n_tiles, q2, 1, s);
+    launch_fold(part, row, fold, n_tiles, q2, 1, s);
   };
   if (step0 == 0) observe(rows, 0);
   const int64_t end = step0 + n_steps;

@@ -94,3 +94,20 @@ def test_steps_between_outputs(q, rep, stride, splits):
     for key in sa:
         assert np.array_equal(sa[key], sb[key]), key
     assert np.array_equal(a.sums(), b.sums())
+
+
+@pytest.mark.parametrize("modes", [32, 33, 65])
+def test_rows_do_not_depend_on_the_buffer(q, modes):
+    """Rows of a many-mode model with a buffer of zeros and one of large numbers:
+    only what the observation has written is added up."""
+    model = wl.random_lvc2(modes, seed=3, scale=0.1)
+    init = wl.sb_init(model, beta=2.0)
+    rows = []
+    for fill in (0, 0x7E):
+        r = q.SpawnRun(q.Model(model), 700, 20_000, 2, 5, precision=q.PREC_FP32_BULK)
+        r.obs_buf.fill_(fill)
+        r.sample(init)
+        r.propagate(8, 0.01, 2)
+        rows.append(r.sums())
+    assert np.isfinite(rows[0]).all()
+    assert np.array_equal(rows[0], rows[1])
