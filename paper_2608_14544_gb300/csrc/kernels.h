@@ -349,13 +349,16 @@ void launch_spawnN_observe32(int ns, const BulkParams& bp, const CoefN& cf, cons
                              int64_t capacity, int64_t n0, int set, double* part,
                              cudaStream_t st);
 // FP32-bulk spawning (two states): sample, steps [step, step + len) of a call that
-// began at step0, family observation.
+// began at step0 (chain: chained steps, spawn_chained32), family observation
+// (starts: the families' starts are there, left by chained steps).
+bool spawn_chained32(int n);
 void launch_spawn_sample32(const DevModel& host, const SampleParams& sp, int64_t capacity, void* buf,
                            cudaStream_t st);
 void launch_spawn_steps32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t capacity,
-                          int64_t n0, int64_t step0, int64_t step, int64_t len, cudaStream_t st);
+                          int64_t n0, int64_t step0, int64_t step, int64_t len, bool chain,
+                          cudaStream_t st);
 void launch_spawn_observe32(const BulkParams& bp, const Coef2& cf, const void* buf, int64_t capacity,
-                            int64_t n0, int set, double* part, cudaStream_t st);
+                            int64_t n0, int set, bool starts, double* part, cudaStream_t st);
 
 // Kernel launches issued by the library (instrumentation).
 void launches_add(int64_t k);

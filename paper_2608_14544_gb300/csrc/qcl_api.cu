@@ -996,6 +996,7 @@ qcl_status qcl_spawn_propagate(const qcl_model* model, const qcl_ensemble_desc* 
   const int64_t n0 = ens->n_traj;
   const bool f32 = ens->precision == QCL_PREC_FP32_BULK;
   const bool f32n = f32 && model->ns > 2;
+  const bool chain = spawn_chained32(model->n);  // (one reading of the option for the call)
   Coef2* cf = nullptr;
   CoefN* cn = nullptr;
   BulkParams bp{};
@@ -1016,18 +1017,28 @@ qcl_status qcl_spawn_propagate(const qcl_model* model, const qcl_ensemble_desc* 
     bp.n = model->n;
     bulk_model_scalars(bp, model->host, dt);
   }
-  auto observe = [&](double* row, int64_t step) {
-    if (f32n)
-      launch_spawnN_observe32(model->ns, bp, *cn, buf, capacity, n0, (int)(step & 1), part, s);
-    else if (f32)
-      launch_spawn_observe32(bp, *cf, buf, capacity, n0, (int)(step & 1), part, s);
-    else if (model->ns > 2)
-      launch_spawnN_observe(model->dev, model->ns, buf, capacity, model->n, n0, (int)(step & 1), part, s);
-    else
-      launch_spawn_observe(model->dev, buf, capacity, model->n, n0, (int)(step & 1), part, s);
-    launch_fold(part, row, fold, n_tiles, q2, 1, s);
+  // output times wait in part's slots and are folded together (a fold after
+  // each took 12 us)
+  int slots = 0;
+  int64_t k_slot = 0;
+  auto flush = [&]() {
+    if (slots > 0) launch_fold(part, rows + (size_t)k_slot * q2, fold, n_tiles, q2, slots, s);
+    slots = 0;
   };
-  if (step0 == 0) observe(rows, 0);
+  auto observe = [&](int64_t k, int64_t step) {
+    if (slots == 0) k_slot = k;
+    double* at = part + (size_t)slots * n_tiles * q2;
+    if (f32n)
+      launch_spawnN_observe32(model->ns, bp, *cn, buf, capacity, n0, (int)(step & 1), at, s);
+    else if (f32)
+      launch_spawn_observe32(bp, *cf, buf, capacity, n0, (int)(step & 1), chain && step > step0, at, s);
+    else if (model->ns > 2)
+      launch_spawnN_observe(model->dev, model->ns, buf, capacity, model->n, n0, (int)(step & 1), at, s);
+    else
+      launch_spawn_observe(model->dev, buf, capacity, model->n, n0, (int)(step & 1), at, s);
+    if (++slots == kChunkOut) flush();
+  };
+  if (step0 == 0) observe(0, 0);
   const int64_t end = step0 + n_steps;
   for (int64_t t = step0; t < end;) {
     // (two states in FP32: the steps up to the next output time at once)
@@ -1037,15 +1048,16 @@ qcl_status qcl_spawn_propagate(const qcl_model* model, const qcl_ensemble_desc* 
       if (f32n)
         launch_spawnN_step32(model->ns, bp, *cn, buf, capacity, n0, step0, t, s);
       else if (f32)
-        launch_spawn_steps32(bp, *cf, buf, capacity, n0, step0, t, len, s);
+        launch_spawn_steps32(bp, *cf, buf, capacity, n0, step0, t, len, chain, s);
       else if (model->ns > 2)
         launch_spawnN_step(model->dev, model->ns, buf, capacity, model->n, n0, step0, t, dt, ens->seed, s);
       else
         launch_spawn_step(model->host, buf, capacity, n0, step0, t, dt, ens->seed, s);
     }
     t += len;
-    if (t % out_stride == 0) observe(rows + (size_t)(t / out_stride) * q2, t);
+    if (t % out_stride == 0) observe(t / out_stride, t);
   }
+  flush();
   delete cf;
   delete cn;
   st = check_launch("spawn step");

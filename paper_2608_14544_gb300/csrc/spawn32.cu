@@ -65,7 +65,12 @@ __global__ void __launch_bounds__(256) k_spawn_sample32(const Sample32 sp, int64
     sh->n_live[1] = 0;
     sh->drop = 0;
   }
+  // the families' starts: an observation finds indexes within the buffer whatever
+  // the steps before it did (a step mismatch moves nothing)
+  int64_t* const fstart = (int64_t*)((char*)buf + L.fstart);
+  if (i == 0) fstart[n0] = n0;
   if (i >= n0) return;
+  fstart[i] = i;
   const Set32 w = set32(buf, L, 0);
   const uint64_t traj = sp.traj_offset + (uint64_t)i;
   float mh;
@@ -285,7 +290,8 @@ __device__ __forceinline__ void add_counts(unsigned int* cnt, bool fires, int64_
 // (`in`) has only to place them and to make the children of the few that fired.
 // So a step is evaluated once; at the ends of an interval between output times,
 // where the set has to hold the plain state, the step is evaluated for its counts
-// and again by the next launch.
+// and again by the next launch.  A launch that writes the plain state also writes
+// the families' starts for the observation (a kernel of its own took 11 us).
 //
 // What bounds it: instruction issue at 1e6 walkers, launch latency below some 1e5
 // (7 us a step).  1e5 initial one-mode walkers growing to 1.57e6 over 400 steps
@@ -298,7 +304,7 @@ __device__ __forceinline__ void add_counts(unsigned int* cnt, bool fires, int64_
 template <int NPL, int KIND, bool DIA, bool FIRST>
 __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
     k_spawn_chain32(const BulkParams bp, const CoefLocal<NPL> cf, const SpawnLayout L, void* buf,
-                    int64_t cap, int64_t step, int in, int out) {
+                    int64_t cap, int64_t n0, int64_t step, int in, int out) {
   __shared__ int wcnt[2][8];
   __shared__ unsigned long long wsum[8];
   EnsHeader* hdr = (EnsHeader*)buf;
@@ -322,6 +328,7 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
   const int64_t per = (groups + gridDim.x - 1) / gridDim.x;
   const int64_t g0 = min((int64_t)blockIdx.x * per, groups), g1 = min(g0 + per, groups);
   const Set32 s = set32(buf, L, src), d = set32(buf, L, src ^ 1);
+  int64_t* const fstart = (int64_t*)((char*)buf + L.fstart);
   SWalker<NPL> x;
   uint64_t id = 0;
   uint32_t fam = 0;
@@ -353,6 +360,7 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       sh->total[kz] = 0;
       sh->n_live[src ^ 1] = drop ? n_live : n_live + total;
+      if (!out) fstart[n0] = drop ? n_live : n_live + total;
       if (drop) atomicOr(&hdr->flags, QCL_FLAG_SPAWN_OVERFLOW);
     }
     if (!drop && g0 < g1) {
@@ -398,6 +406,9 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
         prefix += c;
         if (hop) idc = child_id32(bp.seed, step, id);
         if (!out) {
+          // a family's first walker stays its first: children follow parents
+          const uint32_t left = __shfl_up_sync(0xffffffffu, fam, 1);
+          if (live && (i == 0 || (lane > 0 ? left : s.fam[i - 1]) != fam)) fstart[fam] = pos;
           if (live) put_walker(d, cap, bp.n, pos, x, id, fam);
           if (hop) put_walker(d, cap, bp.n, pos + 1, xc, idc, fam);
         }
@@ -772,12 +783,12 @@ void run_steps32(const BulkParams& bp, const Coef2& c2, void* buf, int64_t cap, 
   const unsigned grid = spawn_grid(cap, per_sm);
   if (step == bp.step0) {
     k_spawn_chain_clear<<<grid, 256, 0, st>>>(buf, cap, bp.n, n0);
-    k_spawn_chain32<NPL, KIND, DIA, true><<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, step, 0, 0);
+    k_spawn_chain32<NPL, KIND, DIA, true><<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, n0, step, 0, 0);
     launches_add(2);
   }
   for (int64_t t = step; t < step + len; ++t)
     k_spawn_chain32<NPL, KIND, DIA, false>
-        <<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, t, t > step, t + 1 < step + len);
+        <<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, n0, t, t > step, t + 1 < step + len);
   launches_add(len);
 }
 
@@ -785,9 +796,9 @@ void run_steps32(const BulkParams& bp, const Coef2& c2, void* buf, int64_t cap, 
 // QCL_OPT_MODES_IN_MEMORY = 1) in memory, three launches a step.
 template <int KIND, bool DIA>
 void dispatch_steps32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t cap, int64_t n0,
-                      int64_t step0, int64_t step, int64_t len, cudaStream_t st) {
+                      int64_t step0, int64_t step, int64_t len, bool chain, cudaStream_t st) {
   const int n = bp.n;
-  if (n > 32 || option_modes_in_memory() == 1) {
+  if (!chain) {
     for (int64_t t = step; t < step + len; ++t) {
       k_spawn_step32<KIND, DIA><<<spawn_grid(cap), 256, 0, st>>>(bp, cf, buf, cap, n0, t);
       launch_spawn_scan(buf, cap, n, n0, QCL_PREC_FP32_BULK, 2, step0, t, st);
@@ -815,16 +826,21 @@ void launch_spawn_sample32(const DevModel& host, const SampleParams& sp, int64_t
   launches_add(1);
 }
 
+bool spawn_chained32(int n) { return n <= 32 && option_modes_in_memory() != 1; }
+
 void launch_spawn_steps32(const BulkParams& bp, const Coef2& cf, void* buf, int64_t capacity,
-                          int64_t n0, int64_t step0, int64_t step, int64_t len, cudaStream_t st) {
-  auto run = [&](auto f) { f(bp, cf, buf, capacity, n0, step0, step, len, st); };
+                          int64_t n0, int64_t step0, int64_t step, int64_t len, bool chain,
+                          cudaStream_t st) {
+  auto run = [&](auto f) { f(bp, cf, buf, capacity, n0, step0, step, len, chain, st); };
   if (bp.repr == QCL_REPR_DIABATIC) run(bp.kind == 0 ? dispatch_steps32<0, true> : dispatch_steps32<1, true>);
   else run(bp.kind == 0 ? dispatch_steps32<0, false> : dispatch_steps32<1, false>);
 }
 
 void launch_spawn_observe32(const BulkParams& bp, const Coef2& cf, const void* buf, int64_t capacity,
-                            int64_t n0, int set, double* part, cudaStream_t st) {
-  launch_spawn_fstart(buf, capacity, bp.n, n0, QCL_PREC_FP32_BULK, 2, set, st);
+                            int64_t n0, int set, bool starts, double* part, cudaStream_t st) {
+  // (starts: chained steps have left the families' starts)
+  if (!starts)
+    launch_spawn_fstart(buf, capacity, bp.n, n0, QCL_PREC_FP32_BULK, 2, set, st);
   const unsigned nf = (unsigned)((n0 + 255) / 256);
   const bool dia = bp.repr == QCL_REPR_DIABATIC;
   if (dia)
