@@ -539,27 +539,6 @@ __device__ __forceinline__ Contrib contrib_factors(const Scal& z, float mm) {
   return o;
 }
 
-// The walker's 16 observable contributions (diabatic rho_ij and adiabatic
-// rho_ab, real and imaginary) with weight mantissa `mm`.
-template <bool DIA>
-__device__ __forceinline__ void contributions(const Scal& z, float mm, float (&v)[16]) {
-  const Contrib c = contrib_factors<DIA>(z, mm);
-  constexpr int other = DIA ? 8 : 0, own = DIA ? 0 : 8;
-  v[other + 0] = c.zr * c.f00;
-  v[other + 1] = c.zi * c.f00;
-  v[other + 2] = c.zr * c.f01;
-  v[other + 3] = c.zi * c.f01;
-  v[other + 4] = c.zr * c.f10;
-  v[other + 5] = c.zi * c.f10;
-  v[other + 6] = c.zr * c.f11;
-  v[other + 7] = c.zi * c.f11;
-#pragma unroll
-  for (int kk = 0; kk < 4; ++kk) {
-    v[own + 2 * kk] = (kk == c.k) ? c.zr : 0.0f;
-    v[own + 1 + 2 * kk] = (kk == c.k) ? c.zi : 0.0f;
-  }
-}
-
 // x 2^ex as a double, exactly (built from the bits for normal x and results in
 // the normal double range; zero, subnormal, non-finite or out-of-range values
 // go through ldexp).

@@ -633,52 +633,91 @@ __global__ void __launch_bounds__(256) k_spawn_scatter32(void* buf, int64_t cap,
   }
 }
 
+// a += x f with the product's own rounding error: the rounded product enters the
+// sum, the exact one its error term.  (Written out: with a fused product in both,
+// as the compiler may have it, the error term misses up to 2^-25 of the terms;
+// this form is exact to 2^-48.)
+__device__ __forceinline__ void add_product(f2& a, float x, float f) {
+  const float s = __fadd_rn(__fmul_rn(x, f), a.hi), bb = __fsub_rn(s, a.hi);
+  const float err = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fmaf_rn(x, f, -bb));
+  a = {s, __fadd_rn(a.lo, err)};
+}
+
 // Family observation: for each family the sum X of its walkers' contributions
-// and X^2.  A warp takes 32 families.  The family shares one power of two (its
-// largest weight exponent), so each walker's contribution is an FP32 value,
-// summed as a compensated FP32 pair per lane (lane l of 32 takes the family's
-// walkers l, l + 32, ...) and then over the lanes by a reduce-scatter of pairs at
-// lane distances 16, 8, 4, 2, 1; X is rebuilt in FP64 from the pair and the
-// exponent exactly.  Lanes without a walker hold zero pairs, which change
-// nothing, so a family of at most w walkers takes w lanes (w = 1, 4, 8 or 16)
-// with the same result, and 32 / w such families go side by side (1e5 families of
-// one walker 88 -> 36 us, of four on average 90 -> 82).  The X of the warp's families then meet in shared memory, where
-// the even lane of a pair adds X, the odd lane X^2, of one quantity over the
-// families in order.  (Accumulating every walker in FP64 kept the FP64 pipe 84 %
-// busy: FP64 is slow on this part.)  The tile's 8 warps are folded by the fixed
-// tree of the observation kernels.
+// and X^2.  A block takes a tile of 256 families.  A family shares one power of
+// two (its largest weight exponent), so each walker's contribution is an FP32
+// value, summed as a compensated FP32 pair per lane (lane l of the family's w
+// takes walkers l, l + w, ...) and then over the lanes by a reduce-scatter of
+// pairs; X is rebuilt in FP64 from the pair and the exponent exactly.  (Accumulating
+// every walker in FP64 kept the FP64 pipe 84 % busy: FP64 is slow on this part.)
+//
+// w = 1 up to 8 walkers, 2 to 16, 4 to 32, 8 to 64, 16 to 128 and 32 beyond:
+// eight walkers a lane, since the reduce-scatter over the lanes and the
+// conversion cost as much as two walkers; and more in a row would leave small
+// ensembles waiting on one lane's chain.  32 / w families go side by side, the
+// block's families ordered by size so that those of a warp are alike and few
+// lanes idle, and the block's warps take such groups in turn, widest first.  The
+// X of the tile's families then meet in shared memory, where the even lane of a
+// pair adds X, the odd lane X^2, of one quantity over a warp's 32 families in
+// order, and the 8 warps are folded by the fixed tree of the observation kernels.
+//
+// Bound by instruction issue, the FP64 pipe (48 operations a family) for small
+// families.  1e5 families growing from 1 to 15.7 walkers: 30 to 93 us, 36 to
+// 160 with one walker a lane and the families of a warp in its own order.
+constexpr int kFamClasses = 8;
 template <int KIND, bool DIA>
 __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp, const Coef2 cf,
                                                          const void* buf, int64_t cap, int64_t n0,
                                                          int set, double* __restrict__ part) {
   __shared__ double red[8][32];
   __shared__ double xs[8][32][17];  // (rows of 17: no bank conflicts between families)
-  __shared__ uint8_t ord[8][32];
+  __shared__ uint8_t ord[256];      // families by class, widest first
+  __shared__ int cnt[kFamClasses][8];
   const SpawnLayout L = SpawnLayout::make(cap, bp.n, n0, QCL_PREC_FP32_BULK);
   const Set32 s = set32((void*)buf, L, set);
   const int64_t* fstart = (const int64_t*)((const char*)buf + L.fstart);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t f0 = (int64_t)blockIdx.x * 256 + warp * 32;
-  // lane l's family and its width class
-  const bool real = f0 + lane < n0;
-  const int64_t mine = real ? fstart[f0 + lane] : 0;
-  const int64_t size = real ? fstart[f0 + lane + 1] - mine : 0;
-  const int cls = !real ? 5 : size <= 1 ? 0 : size <= 4 ? 1 : size <= 8 ? 2 : size <= 16 ? 3 : 4;
-#pragma unroll 1
-  for (int c = 0; c < 5; ++c) {
+  const int64_t f0 = (int64_t)blockIdx.x * 256;
+  // this thread's family and its class: 0 the widest (beyond 128 walkers) to 4
+  // (9 to 16), 5 to 7 one lane (5 to 8, 2 to 4, at most 1)
+  const bool real = f0 + threadIdx.x < n0;
+  const int64_t size = real ? fstart[f0 + threadIdx.x + 1] - fstart[f0 + threadIdx.x] : 0;
+  const int cls = !real ? kFamClasses
+                        : size > 128 ? 0 : size > 64 ? 1 : size > 32 ? 2 : size > 16 ? 3
+                        : size > 8 ? 4 : size > 4 ? 5 : size > 1 ? 6 : 7;
+  unsigned mates = 0;
+#pragma unroll
+  for (int c = 0; c < kFamClasses; ++c) {
     const unsigned in = __ballot_sync(0xffffffffu, cls == c);
-    if (!in) continue;
-    const int w = c == 0 ? 1 : 2 << c, side = 32 / w, count = __popc(in);
-    if (cls == c) ord[warp][__popc(in & ((1u << lane) - 1u))] = (uint8_t)lane;
-    __syncwarp();
+    if (cls == c) mates = in;
+    if (lane == c) cnt[c][warp] = __popc(in);
+  }
+  __syncthreads();
+  if (real) {
+    int at = __popc(mates & ((1u << lane) - 1u));
+    for (int c = 0; c <= cls; ++c)
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (c < cls || k < warp) at += cnt[c][k];
+    ord[at] = (uint8_t)threadIdx.x;
+  }
+  __syncthreads();
+  int first = 0, turn = warp;  // the class's first place in ord, groups until this warp's next
+#pragma unroll 1
+  for (int c = 0; c <= 5; ++c) {
+    int count = 0;
+    for (int c2 = c; c2 < (c == 5 ? kFamClasses : c + 1); ++c2)  // (one-lane classes together)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) count += cnt[c2][k];
+    const int w = 32 >> c, side = 32 / w, groups = (count + side - 1) / side;
     const int sub = lane / w, sl = lane - sub * w;
 #pragma unroll 1
-    for (int at = 0; at < count; at += side) {
+    for (; turn < groups; turn += 8) {
+      const int at = turn * side;
       const bool on = at + sub < count;
-      const int f = ord[warp][on ? at + sub : at];
-      const int64_t j0 = __shfl_sync(0xffffffffu, mine, f);
-      const int64_t len = __shfl_sync(0xffffffffu, size, f);
-      const int64_t j1 = on ? j0 + len : j0;
+      const int f = ord[first + (on ? at + sub : at)];
+      const int64_t j0 = fstart[f0 + f];
+      const int64_t j1 = on ? fstart[f0 + f + 1] : j0;
       int em = -(1 << 28);
       for (int64_t j = j0 + sl; j < j1; j += w)
         if (s.mh[j] != 0.0f) em = max(em, s.me[j]);
@@ -704,12 +743,16 @@ __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp,
         z.ph = {s.ph[j], s.pl[j]};
         const float mh = s.mh[j];
         const float mm = mh == 0.0f ? 0.0f : (mh + s.ml[j]) * pow2i(s.me[j] - em);
-        float v[16];
-        contributions<DIA>(z, mm, v);
+        const Contrib c = contrib_factors<DIA>(z, mm);
+        const float fac[4] = {c.f00, c.f01, c.f10, c.f11};
+        constexpr int other = DIA ? 8 : 0, own = DIA ? 0 : 8;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const f2 t = two_sum(acc[q].hi, v[q]);
-          acc[q] = {t.hi, acc[q].lo + t.lo};
+        for (int q = 0; q < 8; ++q) {
+          const float x = (q & 1) ? c.zi : c.zr;
+          f2& ao = acc[own + q];
+          const f2 t = two_sum(ao.hi, (q >> 1) == c.k ? x : 0.0f);
+          ao = {t.hi, ao.lo + t.lo};
+          add_product(acc[other + q], x, fac[q >> 1]);
         }
       }
       __syncwarp();
@@ -744,15 +787,18 @@ __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp,
 #pragma unroll
       for (int i2 = 0; i2 < 16; ++i2)
         if (on && i2 < keep)
-          xs[warp][f][q0 + i2] = scaled_double(acc[i2].hi, ex) + scaled_double(acc[i2].lo, ex);
+          xs[f >> 5][f & 31][q0 + i2] =
+              scaled_double(acc[i2].hi, ex) + scaled_double(acc[i2].lo, ex);
     }
-    __syncwarp();  // ord is rewritten
+    first += count;
+    turn -= groups;
   }
-  const int nf = (int)max((int64_t)0, min((int64_t)32, n0 - f0));
+  __syncthreads();
+  const int nf = (int)max((int64_t)0, min((int64_t)32, n0 - (f0 + warp * 32)));
   double T = 0.0;
   for (int f = 0; f < nf; ++f) {
     const double X = xs[warp][f][lane >> 1];
-    T = (lane & 1) ? fma(X, X, T) : T + X;
+    T = fma(X, (lane & 1) ? X : 1.0, T);  // (X 1 + T is T + X: one FP64 instruction for both)
   }
   red[warp][(lane & 1) ? 16 + (lane >> 1) : (lane >> 1)] = T;
   __syncthreads();
