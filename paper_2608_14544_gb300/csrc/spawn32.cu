@@ -307,6 +307,12 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
                     int64_t cap, int64_t n0, int64_t step, int in, int out) {
   __shared__ int wcnt[2][8];
   __shared__ unsigned long long wsum[8];
+  if (!FIRST) {
+    // the launch after may bring its blocks in; this one goes on when the launch
+    // before has finished and its writes can be seen
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+  }
   EnsHeader* hdr = (EnsHeader*)buf;
   SpawnHeader* sh = hdr_spawn(buf);
   // (FIRST counts the step itself; otherwise the step after it)
@@ -832,9 +838,21 @@ void run_steps32(const BulkParams& bp, const Coef2& c2, void* buf, int64_t cap, 
     k_spawn_chain32<NPL, KIND, DIA, true><<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, n0, step, 0, 0);
     launches_add(2);
   }
-  for (int64_t t = step; t < step + len; ++t)
-    k_spawn_chain32<NPL, KIND, DIA, false>
-        <<<grid, 256, 0, st>>>(bp, cf, L, buf, cap, n0, t, t > step, t + 1 < step + len);
+  // A step's launch after another step's is a programmatic dependent one: its
+  // blocks come in while the last ones of the step before finish.
+  cudaLaunchAttribute dep{};
+  dep.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  dep.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(256);
+  lc.stream = st;
+  lc.attrs = &dep;
+  for (int64_t t = step; t < step + len; ++t) {
+    lc.numAttrs = t > step ? 1 : 0;
+    cudaLaunchKernelEx(&lc, k_spawn_chain32<NPL, KIND, DIA, false>, bp, cf, L, buf, cap, n0, t,
+                       (int)(t > step), (int)(t + 1 < step + len));
+  }
   launches_add(len);
 }
 
