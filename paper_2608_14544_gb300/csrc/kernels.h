@@ -407,7 +407,8 @@ BulkFn bulk2_split_fn(int n, int kind, int wpt);
 // thread so that every slot gets a tile.  Results do not depend on it.
 int bulk_wpt(BulkFn fn2, int& per_sm, int& n_sm, int64_t n_tiles, const LaunchShape& ls);
 int run_bulk_kernel(BulkFn fn, int& per_sm, int& n_sm, const BulkParams& bp, const Coef2& cf,
-                    void* buf, double* part, const LaunchShape& ls, int wpt, cudaStream_t st);
+                    void* buf, double* part, const LaunchShape& ls, int wpt, cudaStream_t st,
+                    size_t dyn = 0);
 // Occupancy limit (resident blocks per SM) of the two-state bulk kernel that
 // a launch of (n, kind, repr, wpt) would use; 0 if there is none.
 int bulk2_blocks_per_sm(int n, int kind, int repr, int wpt);

@@ -103,7 +103,8 @@ int bulk_wpt(BulkFn fn2, int& per_sm, int& n_sm, int64_t n_tiles, const LaunchSh
 }
 
 int run_bulk_kernel(BulkFn fn, int& per_sm, int& n_sm, const BulkParams& bp, const Coef2& cf,
-                    void* buf, double* part, const LaunchShape& ls, int wpt, cudaStream_t st) {
+                    void* buf, double* part, const LaunchShape& ls, int wpt, cudaStream_t st,
+                    size_t dyn) {
   occupancy(fn, per_sm, n_sm);
   const int bps = (ls.blocks_per_sm > 0 && ls.blocks_per_sm < per_sm) ? ls.blocks_per_sm : per_sm;
   int64_t grid = (int64_t)bps * n_sm;
@@ -111,7 +112,7 @@ int run_bulk_kernel(BulkFn fn, int& per_sm, int& n_sm, const BulkParams& bp, con
   const int64_t units = (bp.n_tiles + wpt - 1) / wpt;
   if (grid > units) grid = units;
   if (grid < 1) grid = 1;
-  fn<<<(unsigned)grid, 256, 0, st>>>(bp, cf, buf, part);
+  fn<<<(unsigned)grid, 256, dyn, st>>>(bp, cf, buf, part);
   launches_add(1);
   return (int)grid;
 }
