@@ -57,7 +57,7 @@ typedef int32_t qcl_status;
 #define QCL_ERR_NOT_FOUND 8    /* unknown request id */
 
 /* Working precision of an ensemble. */
-#define QCL_PREC_FP64 0        /* everything in FP64: one kernel launch per step (comparator) */
+#define QCL_PREC_FP64 0        /* everything in FP64 (comparator) */
 #define QCL_PREC_FP32_BULK 1   /* FP32 Verlet/force/coupling, phase and weight carried as
                                   compensated FP32 pairs, FP64 ensemble reduction;
                                   persistent register-resident kernel */
@@ -191,7 +191,8 @@ qcl_status qcl_sample_initial(const qcl_model* model, const qcl_ensemble_desc* e
  * every observable contribution and of its square, added in a fixed tree
  * (32-walker groups, tiles of qcl_shard_tile_walkers walkers, tiles in index
  * order), so that results do not depend on the launch shape and two calls give
- * the same bits as one.  FP64 ensembles launch one kernel per step; FP32-bulk
+ * the same bits as one.  An FP64 launch runs the steps of up to three output
+ * times or 256 steps (two states), or up to 16 steps (more states); FP32-bulk
  * ensembles run a persistent kernel over the tiles with state held in
  * registers (two-state models of 33..256 modes split each walker's modes over
  * 2 or 4 warps, so their tiles hold 128 or 64 walkers).  N_s-state models
@@ -434,7 +435,8 @@ qcl_status qcl_autotune(qcl_model* model, int64_t probe_walkers, int64_t n_steps
  * ens->n_traj is the number n0 of initial walkers (families) and
  * ens->precision the arithmetic (QCL_PREC_FP64, or QCL_PREC_FP32_BULK: the
  * FP32-bulk walker arithmetic -- compensated phase and weight pairs with a
- * carried exponent -- one step per launch with the state in HBM); capacity is
+ * carried exponent -- with the state in HBM, one launch per step for two
+ * states up to 32 modes and three beyond); capacity is
  * the walker slots the buffer holds (n0 <= capacity <= 2^36).  The observation
  * buffer is sized by qcl_obs_bytes(model, ens, n_out) as for any FP64
  * ensemble; its rows hold, per output, the sums over families of the family
@@ -580,7 +582,8 @@ qcl_status qcl_server_destroy(qcl_server* s);
  *   QCL_OPT_GRID_CAP  cap on the persistent grid (0: SMs x resident blocks);
  *                     results do not depend on it (fixed reduction tree)
  *   QCL_OPT_TIMING    1: record a CUDA event pair on the launching stream around
- *                     every persistent-kernel and FP64 step-kernel launch
+ *                     every persistent-kernel launch and every launch, or
+ *                     group of launches, of FP64 and spawning steps
  *   QCL_OPT_MODES_IN_MEMORY  where the FP32-bulk N_s-state kernels (N_s > 2)
  *                     and the FP32 spawning steps keep R and P: 0 (default)
  *                     the faster form as measured for the model's N_s, mode
@@ -599,8 +602,8 @@ qcl_status qcl_set_option(int32_t key, int64_t value);
 qcl_status qcl_launch_count(int64_t* count, int32_t reset);
 
 /* Device time recorded under QCL_OPT_TIMING for kernel class `which`
- * (0: FP32-bulk persistent kernel, 1: FP64 step kernel): total milliseconds and
- * launch count.  Synchronises the recorded events, then clears them. */
+ * (0: FP32-bulk persistent kernel, 1: FP64 and spawning steps): total
+ * milliseconds and number of recorded pairs.  Synchronises the recorded events, then clears them. */
 qcl_status qcl_kernel_time(int32_t which, double* total_ms, int64_t* launches);
 
 #ifdef __cplusplus
