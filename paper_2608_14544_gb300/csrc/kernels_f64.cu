@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kBlock64) k_steps_f64(const Coef64<NC> c, cons
       const Step64 o = walker_step_f64<NP, NC, KIND, DIA>(
           c, NP > 0 ? R : w.R + i, NP > 0 ? P : w.P + i, nt, d, al, be, phi,
           word_of(wd, (int)(s & 3)) >> 8, deg);
-      m = __dmul_rn(m, o.factor);
+      m = weight64(m, o);
       al ^= o.ev & 1;
       be ^= o.ev >> 1;
       if (DIA) q = (q + o.dq) & 3;

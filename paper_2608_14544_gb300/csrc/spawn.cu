@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(256) k_spawn_step(const Coef64<NC> c, void* bu
       uint8_t* fl = (uint8_t*)((char*)buf + L.flag);
       fl[i] = (uint8_t)flag;
       if (flag) {
-        const double mc = __dmul_rn(m, o.factor);
+        const double mc = weight64(m, o);
         cm[i] = mc;
         cab[i] = (uint16_t)((al ^ (o.ev == 1)) | (((q + o.dq) & 3) << 4) | ((be ^ (o.ev == 2)) << 8));
         if (!isfinite(mc)) {
