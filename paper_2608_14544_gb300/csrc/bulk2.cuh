@@ -430,20 +430,27 @@ __device__ __forceinline__ void sample_walker_f32(const Sample32& sp, uint64_t t
 
 // Threshold T (of 2^24, one event's share) and A_e 2^24 of the first-index event
 // (fac; DIA: of both events) of a spawning walker's test, from its state at
-// R_{n+1}.  Returns whether the gap is degenerate.
+// R_{n+1}.  Returns whether the gap is degenerate.  A walker's test is evaluated
+// up to three times (counted for the next step, taken, and for its child's
+// weight), each in a copy of this code of its own, so every operation whose
+// product the compiler could fuse with a sum is an explicit round-to-nearest one:
+// the copies agree however they are compiled.
 template <int KIND, bool DIA>
 __device__ __forceinline__ bool spawn_rate(const Scal& z, float Av, float Bv, const BulkParams& bp,
                                            uint32_t& T, float& fac) {
+  const float kamp = __fmul_rn(bp.kamp, kP24f), amp = __fmul_rn(bp.amp, kP24f);
   if (DIA) {
-    T = min(__float2uint_rz((bp.kamp * kP24f) * fabsf(Bv)), bp.tmax >> 1);
-    fac = (bp.amp * kP24f) * Bv;
+    T = min(__float2uint_rz(__fmul_rn(kamp, fabsf(Bv))), bp.tmax >> 1);
+    fac = __fmul_rn(amp, Bv);
     return false;
   }
   const bool degen = z.r2 < kDegR2_32;
-  const float gn = (KIND == 1) ? 0.5f * (z.A * Bv - z.B * Av) : (-0.5f * bp.b0) * Av;
-  const float g = degen ? 0.0f : gn * (z.ir * z.ir);
-  T = min(__float2uint_rz((bp.kamp * kP24f) * fabsf(g)), bp.tmax >> 1);
-  fac = (bp.amp * kP24f) * g;
+  const float gn = (KIND == 1)
+                       ? __fmul_rn(0.5f, __fmaf_rn(z.A, Bv, -__fmul_rn(z.B, Av)))
+                       : __fmul_rn(__fmul_rn(-0.5f, bp.b0), Av);
+  const float g = degen ? 0.0f : __fmul_rn(gn, __fmul_rn(z.ir, z.ir));
+  T = min(__float2uint_rz(__fmul_rn(kamp, fabsf(g))), bp.tmax >> 1);
+  fac = __fmul_rn(amp, g);
   return degen;
 }
 
@@ -455,8 +462,8 @@ template <int KIND, bool DIA>
 __device__ __forceinline__ int spawn_event(Scal& z, float w_old, float Av, float Bv, uint32_t word,
                                            const BulkParams& bp, unsigned int& deg, uint32_t& T,
                                            float& fac) {
-  if (DIA) z.ph.lo = __fmaf_rn(bp.hdt_hbar * (z.sb - z.sa), w_old + z.A, z.ph.lo);
-  else z.ph.lo = __fmaf_rn(bp.hdt_hbar * (z.sa - z.sb), w_old + z.r, z.ph.lo);
+  const float dsig = DIA ? __fsub_rn(z.sb, z.sa) : __fsub_rn(z.sa, z.sb);
+  z.ph.lo = __fmaf_rn(__fmul_rn(bp.hdt_hbar, dsig), __fadd_rn(w_old, DIA ? z.A : z.r), z.ph.lo);
   deg += spawn_rate<KIND, DIA>(z, Av, Bv, bp, T, fac) ? 1u : 0u;
   const uint32_t y = word >> 8;
   return y < T ? 1 : (y < 2u * T ? 2 : 0);
@@ -469,9 +476,10 @@ template <bool DIA>
 __device__ __forceinline__ void spawn_child(Scal& child, int ev, uint32_t T, float fac) {
   const bool hop1 = ev == 1;
   // adiabatic: A_1 = -sig_a dt g, A_2 = -sig_b dt g; diabatic: both c = b dt / hbar
-  const float num = DIA ? fac : -(hop1 ? child.sa : child.sb) * fac;
+  const float num = DIA ? fac : __fmul_rn(-(hop1 ? child.sa : child.sb), fac);
   weight_factor(child, num, __uint2float_rn(T));
-  child.m = fast_two_sum(child.m.hi, child.m.lo);
+  const PairV<float> m = fast_two_sum_v(child.m.hi, child.m.lo);
+  child.m = {m.hi, m.lo};
   if (hop1) child.sa = -child.sa;
   else child.sb = -child.sb;
   if (DIA) child.q = (child.q + (hop1 ? 3 : 1)) & 3;

@@ -189,7 +189,7 @@ __device__ __forceinline__ int step_walker(const BulkParams& bp, const CoefLocal
   uint32_t T;
   float fac;
   int ev;
-  const float hsab = bp.hdt * 0.5f * (z.sa + z.sb);
+  const float hsab = __fmul_rn(__fmul_rn(bp.hdt, 0.5f), __fadd_rn(z.sa, z.sb));
   if (DIA) {
     kick_dia<NPL, KIND, CF>(w, cf, hsab);
 #pragma unroll
@@ -205,7 +205,7 @@ __device__ __forceinline__ int step_walker(const BulkParams& bp, const CoefLocal
     kick_dia<NPL, KIND, CF>(w, cf, hsab);
     ev = spawn_event<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, T, fac);
   } else {
-    kick<NPL, KIND, CF>(w, cf, hsab * z.c2, hsab * z.s2);
+    kick<NPL, KIND, CF>(w, cf, __fmul_rn(hsab, z.c2), __fmul_rn(hsab, z.s2));
 #pragma unroll
     for (int j = 0; j < NPL; ++j) w.R[j] = __fmaf_rn(cf.dtm[j], w.P[j], w.R[j]);
     const float r_old = z.r;
@@ -217,7 +217,7 @@ __device__ __forceinline__ int step_walker(const BulkParams& bp, const CoefLocal
       if (KIND == 1) z.B = __fmaf_rn(cf.b[j], w.R[j], z.B);
     }
     closed_form(z);
-    kick<NPL, KIND, CF>(w, cf, hsab * z.c2, hsab * z.s2);
+    kick<NPL, KIND, CF>(w, cf, __fmul_rn(hsab, z.c2), __fmul_rn(hsab, z.s2));
     float Av, Bv;
     coupling_sums<NPL, KIND>(cf, w, Av, Bv);
     ev = spawn_event<KIND, false>(z, r_old, Av, Bv, word, bp, deg, T, fac);
@@ -383,11 +383,13 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
   unsigned int found = 0;  // firing walkers this thread's warp counted (lane 0)
   for (int64_t g = g0; g < g1; ++g) {
     const int64_t i = g * 256 + threadIdx.x;
-    const bool live = i < n_live;
+    bool live = i < n_live;
     if (g > g0) load(g);
     // phase 0: the step itself, of walkers not moved yet; 1: the walkers' next
-    // step; 2: their children's.  One copy of the step's code, so that a walker's
-    // test comes out the same when it is only counted and when it is taken.
+    // step; 2: their children's.  One copy of the step's code, of a third of the
+    // size.  A walker's test comes out the same when it is counted (a call's
+    // first step by the FIRST kernel) and when it is taken, since every rounding
+    // in it is explicit.
     SWalker<NPL> xc;      // the children
     uint64_t idc = 0;
     bool hop = false;
@@ -410,11 +412,19 @@ __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
         }
         pos = i + prefix + before;
         prefix += c;
+        // (with tests that agree with their counts a group's places lie in the buffer;
+        // should they ever differ, nothing is written past its end and the step
+        // counts as one that did not fit)
+        if (min(g * 256 + 256, n_live) + prefix > cap) {
+          if (threadIdx.x == 0) atomicOr(&hdr->flags, QCL_FLAG_SPAWN_OVERFLOW);
+          live = hop = false;
+        }
         if (hop) idc = child_id32(bp.seed, step, id);
         if (!out) {
           // a family's first walker stays its first: children follow parents
           const uint32_t left = __shfl_up_sync(0xffffffffu, fam, 1);
-          if (live && (i == 0 || (lane > 0 ? left : s.fam[i - 1]) != fam)) fstart[fam] = pos;
+          if (live && (i == 0 || (lane > 0 ? left : s.fam[i - 1]) != fam) && (int64_t)fam < n0)
+            fstart[fam] = pos;
           if (live) put_walker(d, cap, bp.n, pos, x, id, fam);
           if (hop) put_walker(d, cap, bp.n, pos + 1, xc, idc, fam);
         }
@@ -501,7 +511,7 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
       uint32_t T;
       float fac;
       int ev;
-      const float hsab = bp.hdt * 0.5f * (z.sa + z.sb);
+      const float hsab = __fmul_rn(__fmul_rn(bp.hdt, 0.5f), __fadd_rn(z.sa, z.sb));
       // P += dt/2 F with the pair's force (kick / kick_dia of one mode)
       auto kick1 = [&](int j, float r, float p, float hu, float hv) {
         p = __fmaf_rn(-cf.hk[j], r, p);
@@ -526,7 +536,7 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
         }
         ev = spawn_event<KIND, true>(z, a_old, 0.0f, z.B, word, bp, deg, T, fac);
       } else {
-        const float hu = hsab * z.c2, hv = hsab * z.s2;
+        const float hu = __fmul_rn(hsab, z.c2), hv = __fmul_rn(hsab, z.s2);
         const float r_old = z.r;
         z.A = bp.a0;
         z.B = bp.b0;
@@ -540,7 +550,7 @@ __global__ void __launch_bounds__(256) k_spawn_step32(const BulkParams bp, const
           s.P[(int64_t)j * cap + i] = p;
         }
         closed_form(z);
-        const float hu2 = hsab * z.c2, hv2 = hsab * z.s2;
+        const float hu2 = __fmul_rn(hsab, z.c2), hv2 = __fmul_rn(hsab, z.s2);
         float Av = 0.0f, Bv = 0.0f;
         for (int j = 0; j < bp.n; ++j) {
           const float r = s.R[(int64_t)j * cap + i];
