@@ -677,10 +677,19 @@ __device__ __forceinline__ void add_product(f2& a, float x, float f) {
 // pair adds X, the odd lane X^2, of one quantity over a warp's 32 families in
 // order, and the 8 warps are folded by the fixed tree of the observation kernels.
 //
+// A family of more than kFamWide walkers is taken by the whole block (a walker of
+// 256 a lane, the warps' pairs added in order), so that the few large families of
+// a model whose walkers multiply near a crossing do not leave the launch waiting
+// for one warp.  200000 families of 13.9 walkers on average, the largest tens of
+// thousands, 16 modes, an output: 1518 us by one warp a family, 338, 324 and 299
+// with the line at 1024, 512 and 256; families without such a tail are unchanged.
+// At 512 the block's eight reductions weigh as much as its sixteen walkers a warp.
+//
 // Bound by instruction issue, the FP64 pipe (48 operations a family) for small
 // families.  1e5 families growing from 1 to 15.7 walkers: 30 to 93 us, 36 to
 // 160 with one walker a lane and the families of a warp in its own order.
-constexpr int kFamClasses = 8;
+constexpr int kFamClasses = 9;
+constexpr int64_t kFamWide = 512;
 template <int KIND, bool DIA>
 __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp, const Coef2 cf,
                                                          const void* buf, int64_t cap, int64_t n0,
@@ -689,18 +698,21 @@ __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp,
   __shared__ double xs[8][32][17];  // (rows of 17: no bank conflicts between families)
   __shared__ uint8_t ord[256];      // families by class, widest first
   __shared__ int cnt[kFamClasses][8];
+  __shared__ int wide_em[8];        // a family of the whole block: its warps' exponents
+  __shared__ f2 wide_sum[8][16];    // and sums
   const SpawnLayout L = SpawnLayout::make(cap, bp.n, n0, QCL_PREC_FP32_BULK);
   const Set32 s = set32((void*)buf, L, set);
   const int64_t* fstart = (const int64_t*)((const char*)buf + L.fstart);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t f0 = (int64_t)blockIdx.x * 256;
-  // this thread's family and its class: 0 the widest (beyond 128 walkers) to 4
-  // (9 to 16), 5 to 7 one lane (5 to 8, 2 to 4, at most 1)
+  // this thread's family and its class: 0 for the whole block, 1 (beyond 128
+  // walkers) to 5 (9 to 16) for 32 to 2 lanes, 6 to 8 one lane (5 to 8, 2 to 4, at
+  // most 1)
   const bool real = f0 + threadIdx.x < n0;
   const int64_t size = real ? fstart[f0 + threadIdx.x + 1] - fstart[f0 + threadIdx.x] : 0;
   const int cls = !real ? kFamClasses
-                        : size > 128 ? 0 : size > 64 ? 1 : size > 32 ? 2 : size > 16 ? 3
-                        : size > 8 ? 4 : size > 4 ? 5 : size > 1 ? 6 : 7;
+                        : size > kFamWide ? 0 : size > 128 ? 1 : size > 64 ? 2 : size > 32 ? 3
+                        : size > 16 ? 4 : size > 8 ? 5 : size > 4 ? 6 : size > 1 ? 7 : 8;
   unsigned mates = 0;
 #pragma unroll
   for (int c = 0; c < kFamClasses; ++c) {
@@ -718,11 +730,111 @@ __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp,
     ord[at] = (uint8_t)threadIdx.x;
   }
   __syncthreads();
-  int first = 0, turn = warp;  // the class's first place in ord, groups until this warp's next
+  // the sum over family f (of the tile) by the w lanes of which this one is `sl`
+  // (WIDE: by the whole block); lanes without a family (on false) only take part
+  auto family = [&](auto wide, int f, bool on, int w, int sl) {
+    constexpr bool WIDE = decltype(wide)::value;
+    const int off0 = WIDE ? threadIdx.x : sl, step = WIDE ? 256 : w;
+    const int64_t j0 = fstart[f0 + f];
+    const int64_t j1 = on ? fstart[f0 + f + 1] : j0;
+    int em = -(1 << 28);
+    for (int64_t j = j0 + off0; j < j1; j += step)
+      if (s.mh[j] != 0.0f) em = max(em, s.me[j]);
+    for (int off = w >> 1; off > 0; off >>= 1)
+      em = max(em, __shfl_xor_sync(0xffffffffu, em, off));
+    if constexpr (WIDE) {
+      if (lane == 0) wide_em[warp] = em;
+      __syncthreads();
+      for (int k = 0; k < 8; ++k) em = max(em, wide_em[k]);
+    }
+    f2 acc[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) acc[q] = {0.0f, 0.0f};
+    for (int64_t j = j0 + off0; j < j1; j += step) {
+      Scal z;
+      z.A = bp.a0;
+      z.B = bp.b0;
+      for (int m = 0; m < bp.n; ++m) {
+        const float r = s.R[(int64_t)m * cap + j];
+        z.A = __fmaf_rn(cf.a[m], r, z.A);
+        if (KIND == 1) z.B = __fmaf_rn(cf.b[m], r, z.B);
+      }
+      closed_form(z);
+      const uint32_t ab = s.ab[j];
+      z.sa = sgn(ab & 0xf);
+      z.sb = sgn((ab >> 8) & 0xf);
+      z.q = DIA ? (int)((ab >> 4) & 3u) : 0;
+      z.ph = {s.ph[j], s.pl[j]};
+      const float mh = s.mh[j];
+      const float mm = mh == 0.0f ? 0.0f : (mh + s.ml[j]) * pow2i(s.me[j] - em);
+      const Contrib c = contrib_factors<DIA>(z, mm);
+      const float fac[4] = {c.f00, c.f01, c.f10, c.f11};
+      constexpr int other = DIA ? 8 : 0, own = DIA ? 0 : 8;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float x = (q & 1) ? c.zi : c.zr;
+        f2& ao = acc[own + q];
+        const f2 t = two_sum(ao.hi, (q >> 1) == c.k ? x : 0.0f);
+        ao = {t.hi, ao.lo + t.lo};
+        add_product(acc[other + q], x, fac[q >> 1]);
+      }
+    }
+    __syncwarp();
+    // reduce-scatter of the pairs: at the step with offset `off`, the lane with
+    // that bit set keeps the upper half of its values (q0: the first it keeps)
+    int q0 = 0, keep = 16, off = w >> 1;
+#pragma unroll
+    for (int half = 8; half >= 1; half >>= 1) {
+      if (off > 0) {
+        const bool upper = (lane & off) != 0;
+#pragma unroll
+        for (int i2 = 0; i2 < half; ++i2) {
+          const f2 snd = upper ? acc[i2] : acc[half + i2];
+          const f2 kp = upper ? acc[half + i2] : acc[i2];
+          const float rh = __shfl_xor_sync(0xffffffffu, snd.hi, off);
+          const float rl = __shfl_xor_sync(0xffffffffu, snd.lo, off);
+          const f2 t = two_sum(kp.hi, rh);
+          acc[i2] = {t.hi, t.lo + (kp.lo + rl)};
+        }
+        q0 += upper ? half : 0;
+        keep = half;
+        off >>= 1;
+      }
+    }
+    if (off > 0) {  // (w = 32: lanes 2q and 2q + 1 both end with quantity q)
+      const float rh = __shfl_xor_sync(0xffffffffu, acc[0].hi, 1);
+      const float rl = __shfl_xor_sync(0xffffffffu, acc[0].lo, 1);
+      const f2 t = two_sum(acc[0].hi, rh);
+      acc[0] = {t.hi, t.lo + (acc[0].lo + rl)};
+    }
+    const int ex = (em < -(1 << 27)) ? 0 : em;
+    if constexpr (WIDE) {  // the warps' sums, in order
+      if (!(lane & 1)) wide_sum[warp][lane >> 1] = acc[0];
+      __syncthreads();
+      if (threadIdx.x < 16) {
+        f2 t = wide_sum[0][threadIdx.x];
+        for (int k = 1; k < 8; ++k) {
+          const f2 x = wide_sum[k][threadIdx.x], u = two_sum(t.hi, x.hi);
+          t = {u.hi, u.lo + (t.lo + x.lo)};
+        }
+        xs[f >> 5][f & 31][threadIdx.x] = scaled_double(t.hi, ex) + scaled_double(t.lo, ex);
+      }
+    } else {
+#pragma unroll
+      for (int i2 = 0; i2 < 16; ++i2)
+        if (on && i2 < keep)
+          xs[f >> 5][f & 31][q0 + i2] =
+              scaled_double(acc[i2].hi, ex) + scaled_double(acc[i2].lo, ex);
+    }
+  };
+  int first = 0;  // the class's first place in ord
+  for (int k = 0; k < 8; ++k) first += cnt[0][k];
+  for (int k = 0; k < first; ++k) family(std::true_type{}, ord[k], true, 32, lane);
+  int turn = warp;  // groups until this warp's next
 #pragma unroll 1
   for (int c = 0; c <= 5; ++c) {
     int count = 0;
-    for (int c2 = c; c2 < (c == 5 ? kFamClasses : c + 1); ++c2)  // (one-lane classes together)
+    for (int c2 = c + 1; c2 < (c == 5 ? kFamClasses : c + 2); ++c2)  // (one-lane classes together)
 #pragma unroll
       for (int k = 0; k < 8; ++k) count += cnt[c2][k];
     const int w = 32 >> c, side = 32 / w, groups = (count + side - 1) / side;
@@ -731,80 +843,7 @@ __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp,
     for (; turn < groups; turn += 8) {
       const int at = turn * side;
       const bool on = at + sub < count;
-      const int f = ord[first + (on ? at + sub : at)];
-      const int64_t j0 = fstart[f0 + f];
-      const int64_t j1 = on ? fstart[f0 + f + 1] : j0;
-      int em = -(1 << 28);
-      for (int64_t j = j0 + sl; j < j1; j += w)
-        if (s.mh[j] != 0.0f) em = max(em, s.me[j]);
-      for (int off = w >> 1; off > 0; off >>= 1)
-        em = max(em, __shfl_xor_sync(0xffffffffu, em, off));
-      f2 acc[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) acc[q] = {0.0f, 0.0f};
-      for (int64_t j = j0 + sl; j < j1; j += w) {
-        Scal z;
-        z.A = bp.a0;
-        z.B = bp.b0;
-        for (int m = 0; m < bp.n; ++m) {
-          const float r = s.R[(int64_t)m * cap + j];
-          z.A = __fmaf_rn(cf.a[m], r, z.A);
-          if (KIND == 1) z.B = __fmaf_rn(cf.b[m], r, z.B);
-        }
-        closed_form(z);
-        const uint32_t ab = s.ab[j];
-        z.sa = sgn(ab & 0xf);
-        z.sb = sgn((ab >> 8) & 0xf);
-        z.q = DIA ? (int)((ab >> 4) & 3u) : 0;
-        z.ph = {s.ph[j], s.pl[j]};
-        const float mh = s.mh[j];
-        const float mm = mh == 0.0f ? 0.0f : (mh + s.ml[j]) * pow2i(s.me[j] - em);
-        const Contrib c = contrib_factors<DIA>(z, mm);
-        const float fac[4] = {c.f00, c.f01, c.f10, c.f11};
-        constexpr int other = DIA ? 8 : 0, own = DIA ? 0 : 8;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float x = (q & 1) ? c.zi : c.zr;
-          f2& ao = acc[own + q];
-          const f2 t = two_sum(ao.hi, (q >> 1) == c.k ? x : 0.0f);
-          ao = {t.hi, ao.lo + t.lo};
-          add_product(acc[other + q], x, fac[q >> 1]);
-        }
-      }
-      __syncwarp();
-      // reduce-scatter of the pairs: at the step with offset `off`, the lane with
-      // that bit set keeps the upper half of its values (q0: the first it keeps)
-      int q0 = 0, keep = 16, off = w >> 1;
-#pragma unroll
-      for (int half = 8; half >= 1; half >>= 1) {
-        if (off > 0) {
-          const bool upper = (lane & off) != 0;
-#pragma unroll
-          for (int i2 = 0; i2 < half; ++i2) {
-            const f2 snd = upper ? acc[i2] : acc[half + i2];
-            const f2 kp = upper ? acc[half + i2] : acc[i2];
-            const float rh = __shfl_xor_sync(0xffffffffu, snd.hi, off);
-            const float rl = __shfl_xor_sync(0xffffffffu, snd.lo, off);
-            const f2 t = two_sum(kp.hi, rh);
-            acc[i2] = {t.hi, t.lo + (kp.lo + rl)};
-          }
-          q0 += upper ? half : 0;
-          keep = half;
-          off >>= 1;
-        }
-      }
-      if (off > 0) {  // (w = 32: lanes 2q and 2q + 1 both end with quantity q)
-        const float rh = __shfl_xor_sync(0xffffffffu, acc[0].hi, 1);
-        const float rl = __shfl_xor_sync(0xffffffffu, acc[0].lo, 1);
-        const f2 t = two_sum(acc[0].hi, rh);
-        acc[0] = {t.hi, t.lo + (acc[0].lo + rl)};
-      }
-      const int ex = (em < -(1 << 27)) ? 0 : em;
-#pragma unroll
-      for (int i2 = 0; i2 < 16; ++i2)
-        if (on && i2 < keep)
-          xs[f >> 5][f & 31][q0 + i2] =
-              scaled_double(acc[i2].hi, ex) + scaled_double(acc[i2].lo, ex);
+      family(std::false_type{}, ord[first + (on ? at + sub : at)], on, w, sl);
     }
     first += count;
     turn -= groups;
