@@ -667,10 +667,15 @@ __device__ __forceinline__ void add_product(f2& a, float x, float f) {
 // pairs; X is rebuilt in FP64 from the pair and the exponent exactly.  (Accumulating
 // every walker in FP64 kept the FP64 pipe 84 % busy: FP64 is slow on this part.)
 //
-// w = 1 up to 8 walkers, 2 to 16, 4 to 32, 8 to 64, 16 to 128 and 32 beyond:
-// eight walkers a lane, since the reduce-scatter over the lanes and the
-// conversion cost as much as two walkers; and more in a row would leave small
-// ensembles waiting on one lane's chain.  32 / w families go side by side, the
+// w = 1 up to `per` walkers, twice as many lanes for every doubling, 32 beyond 16
+// `per`.  per = 8 up to 24 modes, since the reduce-scatter over the lanes and the
+// conversion cost as much as two walkers, and more in a row would leave small
+// ensembles waiting on one lane's chain; 4 up to 64 modes and 1 beyond, where a
+// walker's own loads outweigh the reduction and lanes of one family read
+// neighbouring walkers.  An output of 200000 families by 8, 4, 2 and 1: 13.8
+// walkers of 32 modes 411, 338, 348 and 378 us, 5.2 of 40 modes 273, 230, 203 and
+// 215, 5.4 of 100 modes 689, 567, 492 and 458; of 16 modes 203, 206, 223 and 244.
+// 32 / w families go side by side, the
 // block's families ordered by size so that those of a warp are alike and few
 // lanes idle, and the block's warps take such groups in turn, widest first.  The
 // X of the tile's families then meet in shared memory, where the even lane of a
@@ -689,11 +694,12 @@ __device__ __forceinline__ void add_product(f2& a, float x, float f) {
 // families.  1e5 families growing from 1 to 15.7 walkers: 30 to 93 us, 36 to
 // 160 with one walker a lane and the families of a warp in its own order.
 constexpr int kFamClasses = 9;
-constexpr int64_t kFamWide = 512;
+constexpr int64_t kFamWide = 512;  // (half of it above 64 modes, `per` = 1)
 template <int KIND, bool DIA>
 __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp, const Coef2 cf,
                                                          const void* buf, int64_t cap, int64_t n0,
-                                                         int set, double* __restrict__ part) {
+                                                         int set, int per,
+                                                         double* __restrict__ part) {
   __shared__ double red[8][32];
   __shared__ double xs[8][32][17];  // (rows of 17: no bank conflicts between families)
   __shared__ uint8_t ord[256];      // families by class, widest first
@@ -705,14 +711,16 @@ __global__ void __launch_bounds__(256, 4) k_spawn_observe32(const BulkParams bp,
   const int64_t* fstart = (const int64_t*)((const char*)buf + L.fstart);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t f0 = (int64_t)blockIdx.x * 256;
-  // this thread's family and its class: 0 for the whole block, 1 (beyond 128
-  // walkers) to 5 (9 to 16) for 32 to 2 lanes, 6 to 8 one lane (5 to 8, 2 to 4, at
-  // most 1)
+  // this thread's family and its class: 0 for the whole block, 1 (beyond 16 `per`
+  // walkers) to 5 (beyond `per`) for 32 to 2 lanes, 6 to 8 one lane (beyond half of
+  // it, 2 or more, at most 1)
   const bool real = f0 + threadIdx.x < n0;
   const int64_t size = real ? fstart[f0 + threadIdx.x + 1] - fstart[f0 + threadIdx.x] : 0;
   const int cls = !real ? kFamClasses
-                        : size > kFamWide ? 0 : size > 128 ? 1 : size > 64 ? 2 : size > 32 ? 3
-                        : size > 16 ? 4 : size > 8 ? 5 : size > 4 ? 6 : size > 1 ? 7 : 8;
+                        : size > (per > 1 ? kFamWide : kFamWide / 2) ? 0
+                        : size > 16 * per ? 1 : size > 8 * per ? 2 : size > 4 * per ? 3
+                        : size > 2 * per ? 4 : size > per ? 5 : size > (per >> 1) ? 6
+                        : size > 1 ? 7 : 8;
   unsigned mates = 0;
 #pragma unroll
   for (int c = 0; c < kFamClasses; ++c) {
@@ -956,12 +964,13 @@ void launch_spawn_observe32(const BulkParams& bp, const Coef2& cf, const void* b
     launch_spawn_fstart(buf, capacity, bp.n, n0, QCL_PREC_FP32_BULK, 2, set, st);
   const unsigned nf = (unsigned)((n0 + 255) / 256);
   const bool dia = bp.repr == QCL_REPR_DIABATIC;
+  const int per = bp.n <= 24 ? 8 : (bp.n <= 64 ? 4 : 1);  // walkers a lane
   if (dia)
     (bp.kind == 0 ? k_spawn_observe32<0, true> : k_spawn_observe32<1, true>)
-        <<<nf, 256, 0, st>>>(bp, cf, buf, capacity, n0, set, part);
+        <<<nf, 256, 0, st>>>(bp, cf, buf, capacity, n0, set, per, part);
   else
     (bp.kind == 0 ? k_spawn_observe32<0, false> : k_spawn_observe32<1, false>)
-        <<<nf, 256, 0, st>>>(bp, cf, buf, capacity, n0, set, part);
+        <<<nf, 256, 0, st>>>(bp, cf, buf, capacity, n0, set, per, part);
   launches_add(1);
 }
 
