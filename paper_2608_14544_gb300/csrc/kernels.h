@@ -371,6 +371,17 @@ int64_t launch_steps_f64(const DevModel& host, void* buf, int64_t nt, int64_t st
                          int64_t end, int32_t stride, bool obs_first, double dt, uint64_t seed,
                          uint64_t traj_off, double* part, int* outs, cudaStream_t st);
 
+// Allows kernel fn `bytes` of dynamic shared memory on the current device.  The
+// limit belongs to a device, so it is set before every launch that may pass 48 KB,
+// and to the same value for every launch of a kernel, so that threads launching
+// other sizes do not lower it under each other.  False when it is refused: the
+// launch is left out, and the caller's check of the launch reports the error.
+template <typename Fn>
+inline bool allow_dynamic_shared(Fn fn, size_t bytes) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) ==
+         cudaSuccess;
+}
+
 // Launch shape of a persistent bulk launch; the results do not depend on it.
 struct LaunchShape {
   int wpt = 0;            // walkers per thread, 1 or 2 (0: the default for the mode count)

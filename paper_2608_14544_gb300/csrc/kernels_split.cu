@@ -649,9 +649,7 @@ int run_split(const BulkParams& bp, const Coef2& cf, void* buf, double* part,
     if (wpt == 2) wpt = bulk_wpt(split_fn<NPL, L, KIND, 2>(), per_sm[1], n_sm[1], bp.n_tiles, ls);
     if (wpt == 2) {
       constexpr size_t stage = split_stage_bytes<NPL, L, 2>();
-      static const cudaError_t set = cudaFuncSetAttribute(
-          split_fn<NPL, L, KIND, 2>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage);
-      (void)set;  // (a refusal shows as the launch's own error)
+      if (stage > 0 && !allow_dynamic_shared(split_fn<NPL, L, KIND, 2>(), stage)) return 1;
       return run_bulk_kernel(split_fn<NPL, L, KIND, 2>(), per_sm[1], n_sm[1], bp, cf, buf, part,
                              ls, 2, st, stage);
     }

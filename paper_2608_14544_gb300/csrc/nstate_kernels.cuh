@@ -64,14 +64,7 @@ struct NStateOps {
     size_t dyn = 0;
     if constexpr (NPL == 0) {
       dyn = ModeRow<NS>::bytes(bp.n);
-      static std::mutex mu;
-      static size_t dyn_set = 0;
-      std::lock_guard<std::mutex> lock(mu);
-      if (dyn > dyn_set) {
-        cudaFuncSetAttribute(k_spawnN_step32<NS, NPL>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        dyn_set = dyn;
-      }
+      if (!allow_dynamic_shared(k_spawnN_step32<NS, NPL>, ModeRow<NS>::bytes(kMaxN))) return;
     }
     k_spawnN_step32<NS, NPL><<<spawn_grid(cap), 256, dyn, st>>>(bp, cf, buf, cap, n0, step);
   }
@@ -107,35 +100,34 @@ struct NStateOps {
   template <int NPL, int WPT = 1, int NM = 0, int SM = 0>
   static int bulk_npl(const BulkParams& bp, const CoefN& cf, const ModeHost& mh, void* buf,
                       double* part, int grid_cap, cudaStream_t st) {
-    // (occupancy cached per kernel and table size: [0] adiabatic, [1] diabatic;
-    // NPL = 0: the mode table in dynamic shared memory)
+    // (occupancy cached per kernel: [0] adiabatic, [1] diabatic; NPL = 0: the mode
+    // table, or R and P, in dynamic shared memory, at most dyn_max of it)
     static int per_sm[2] = {-1, -1}, n_sm[2] = {0, 0};
-    static size_t dyn_at[2] = {0, 0};
     const size_t dyn = NPL != 0  ? 0
                        : NM == 0 ? ModeRow<NS>::bytes(bp.n)
                                  : (size_t)SM * bp.n * 128 * sizeof(float);
+    const size_t dyn_max = NM == 0 ? ModeRow<NS>::bytes(kMaxN) : (size_t)64 * 128 * sizeof(float);
     if constexpr (NM == 0) {
       if (bp.repr == QCL_REPR_DIABATIC)
-        return launch_persistent(k_bulkN_dia<NS, NPL>, per_sm[1], n_sm[1], dyn_at[1], bp, grid_cap,
-                                 1, dyn, st, bp, cf, buf, part);
+        return launch_persistent(k_bulkN_dia<NS, NPL>, per_sm[1], n_sm[1], bp, grid_cap, 1, dyn,
+                                 dyn_max, st, bp, cf, buf, part);
     }
     if constexpr (NPL == 0 && NM == 0 && NS <= 4) {
       return 0;  // (adiabatic models of N_s <= 4 take NM > 0)
     } else {
       CoefMem<NS, NM> cm;
       if constexpr (NM > 0) make_coef_mem(mh, bp.n, cm);
-      return launch_persistent(k_bulkN<NS, NPL, WPT, NM, SM>, per_sm[0], n_sm[0], dyn_at[0], bp,
-                               grid_cap, WPT, dyn, st, bp, cf, buf, part, cm);
+      return launch_persistent(k_bulkN<NS, NPL, WPT, NM, SM>, per_sm[0], n_sm[0], bp,
+                               grid_cap, WPT, dyn, dyn_max, st, bp, cf, buf, part, cm);
     }
   }
   // one persistent grid: the occupancy limit of resident blocks on every SM
   // (capped), at most one block per WPT tiles
-  // (dyn > 0, the modes-in-memory kernels: the shared-memory limit only grows
-  // and the occupancy is computed for this call's table, under a lock, so
-  // that threads launching models of different mode counts do not race)
+  // (dyn > 0, the modes-in-memory kernels: the occupancy is computed for this
+  // call's table)
   template <typename Fn, typename... Args>
-  static int launch_persistent(Fn fn, int& per_sm, int& n_sm, size_t& dyn_at, const BulkParams& bp,
-                               int grid_cap, int WPT, size_t dyn, cudaStream_t st,
+  static int launch_persistent(Fn fn, int& per_sm, int& n_sm, const BulkParams& bp, int grid_cap,
+                               int WPT, size_t dyn, size_t dyn_max, cudaStream_t st,
                                const Args&... args) {
     int blocks = per_sm;
     if (dyn > 0) {
@@ -146,10 +138,7 @@ struct NStateOps {
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
       }
-      if (dyn > dyn_at) {
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        dyn_at = dyn;
-      }
+      if (!allow_dynamic_shared(fn, dyn_max)) return 1;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, 128, dyn) != cudaSuccess ||
           blocks < 1)
         blocks = 1;
