@@ -429,7 +429,9 @@ const char* bulk2_variant(int n, int kind);
 // N_s-state initial sample: FP64 (dm, sp) or FP32 bulk (s32).
 void launch_sampleN(const DevModel* dm, const SampleParams& sp, const SampleN32* s32, void* buf,
                     int precision, cudaStream_t st);
-// Steps [step, step + len) of an N_s-state ensemble (one launch).
+// Steps [step, step + len) of an N_s-state ensemble (one launch), and the most that
+// one should take.
+int32_t steps_per_launchN_f64(int ns, int n, int repr, int64_t nt);
 void launch_stepsN_f64(const DevModel* dm, int repr, int ns, void* buf, int64_t nt, int n,
                        int64_t step0, int64_t step, int32_t len, double dt, uint64_t seed,
                        uint64_t traj_off, cudaStream_t st);

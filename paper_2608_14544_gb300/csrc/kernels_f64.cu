@@ -153,18 +153,30 @@ void launch_sample_f64(const DevModel* dm, const SampleParams& sp, void* buf, cu
   launches_add(1);
 }
 
+// The steps of a launch: at most 256, and as many as keep it near a quarter of a
+// second, since work on other streams waits for its blocks to be handed out.  A
+// step takes up to 35 ps for each walker and mode and as much again for two modes
+// (2e5 walkers: 20 ps with 256 modes of the spin-boson form, 35 of the general one;
+// 1.1 of 3 with one mode).  What a launch adds, a load and a store of the walkers
+// and one decomposition, is small against the ten steps and more that all but
+// the largest ensembles take.
+static int64_t steps_per_launch(int64_t nt, int n) {
+  const double steps = 0.25 / (35e-12 * (double)nt * (double)(n + 2));
+  return steps >= 256.0 ? 256 : std::max<int64_t>((int64_t)steps, 1);
+}
+
 // Steps from `step` with at most kOuts64 output times: returns the steps taken
-// (at most 256, so that a launch of 1e7 walkers stays below a second; 0 with
-// obs_first alone at the end) and leaves the tile partials of *outs output times
-// in part's first slots.  The group sums lie behind them in the same array (its
-// kChunkOut slots hold 9 kOuts64 of a tile's 32 doubles).
+// (0 with obs_first alone at the end) and leaves the tile partials of *outs output
+// times in part's first slots.  The group sums lie behind them in the same array
+// (its kChunkOut slots hold 9 kOuts64 of a tile's 32 doubles).
 int64_t launch_steps_f64(const DevModel& host, void* buf, int64_t nt, int64_t step0, int64_t step,
                          int64_t end, int32_t stride, bool obs_first, double dt, uint64_t seed,
                          uint64_t traj_off, double* part, int* outs, cudaStream_t st) {
   static_assert(9 * kOuts64 <= kChunkOut, "room for the group sums");
   const int64_t next = (step / stride + 1) * stride;  // the first output time after step
   const int room = kOuts64 - (obs_first ? 1 : 0);
-  const int64_t e = std::min(std::min(end, step + 256), next + (int64_t)(room - 1) * stride);
+  const int64_t e = std::min(std::min(end, step + steps_per_launch(nt, host.n)),
+                             next + (int64_t)(room - 1) * stride);
   *outs = (obs_first ? 1 : 0) + (e >= next ? (int)((e - next) / stride) + 1 : 0);
   const int64_t n_tiles = (nt + kTile - 1) / kTile, n_groups = (nt + 31) / 32;
   double* groups = part + (size_t)kOuts64 * n_tiles * 32;

@@ -50,6 +50,19 @@ void launch_sampleN(const DevModel* dm, const SampleParams& sp, const SampleN32*
   launches_add(1);
 }
 
+// The steps of a launch: at most 16, which leaves the decomposition that a launch
+// repeats at 3 % of it, and as many as keep it near a quarter of a second, since
+// work on other streams waits for its blocks to be handed out.  An adiabatic step
+// takes about 0.03 ns N_s^3 (n + 7) for each walker, a diabatic one
+// 0.012 N_s^2 (n + 12): 0.8 to 1.5 and 1.1 to 2.1 times what 2e4 and 1e5 walkers
+// of 3 to 8 states and 2 to 40 modes take.
+int32_t steps_per_launchN_f64(int ns, int n, int repr, int64_t nt) {
+  const double s2 = (double)(ns * ns);
+  const double ns_step = repr == QCL_REPR_DIABATIC ? 0.012 * s2 * (n + 12) : 0.03 * s2 * ns * (n + 7);
+  const double steps = 0.25e9 / (ns_step * (double)nt);
+  return steps >= 16.0 ? 16 : (steps > 1.0 ? (int32_t)steps : 1);
+}
+
 void launch_stepsN_f64(const DevModel* dm, int repr, int ns, void* buf, int64_t nt, int n,
                        int64_t step0, int64_t step, int32_t len, double dt, uint64_t seed,
                        uint64_t traj_off, cudaStream_t st) {

@@ -523,10 +523,10 @@ qcl_status qcl_propagate(const qcl_model* model, const qcl_ensemble_desc* ens, v
         if (++slots == kChunkOut) flush();
       };
       if (step0 == 0) observe(0);
+      const int32_t most = steps_per_launchN_f64(ns, model->n, model->host.repr, nt);
       for (int64_t t = step0; t < end;) {
-        // up to the next output time, at most 16 steps (a launch of 1e6 walkers then
-        // stays below a second)
-        const int64_t len = std::min<int64_t>(std::min<int64_t>(end, (t / out_stride + 1) * out_stride) - t, 16);
+        // (up to the next output time)
+        const int64_t len = std::min<int64_t>(std::min<int64_t>(end, (t / out_stride + 1) * out_stride) - t, most);
         {
           TimedLaunch tl(1, s);
           launch_stepsN_f64(model->dev, model->host.repr, ns, ens_buf, nt, model->n, step0, t, (int32_t)len, dt, ens->seed, ens->traj_id_offset, s);

@@ -93,3 +93,21 @@ def test_spawning_on_a_second_device(fake, ns, n):
             assert lib.fake_max_dyn(b"k_spawnN_step32") > 0
     finally:
         lib.cudaSetDevice(0)
+
+
+@pytest.mark.parametrize("ns,n,rep,walkers,steps,least,most", [
+    (2, 1, "adiabatic", 10_000, 600, 3, 3), (2, 3, "adiabatic", 1_000_000, 512, 2, 2),
+    (2, 256, "adiabatic", 10_000_000, 256, 100, 256), (2, 100, "diabatic", 3_000_000, 256, 5, 64),
+    (4, 6, "adiabatic", 20_000, 32, 2, 2), (4, 6, "diabatic", 1_000_000, 32, 2, 2),
+    (8, 256, "adiabatic", 1_000_000, 32, 32, 32), (4, 40, "adiabatic", 1_000_000, 32, 8, 32)])
+def test_fp64_launches_follow_the_work_of_a_step(fake, ns, n, rep, walkers, steps, least, most):
+    """Small solves take many steps a launch; one of 1e7 walkers and 256 modes,
+    whose step takes a tenth of a second, takes few."""
+    q, lib = fake
+    model = wl.random_lvc2(n, 3, 0.3) if ns == 2 else _lvc(ns, n)
+    r = q.Run(q.Model(dict(model, repr=rep)), walkers, 1, q.PREC_FP64, 2)
+    lib.fake_reset()
+    r.propagate(steps, 0.01, 1000)
+    kernel = b"k_steps_f64" if ns == 2 else (b"k_stepsN_dia_f64" if rep == "diabatic"
+                                            else b"k_stepsN_f64")
+    assert least <= lib.fake_count(kernel) <= most
