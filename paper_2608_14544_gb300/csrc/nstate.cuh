@@ -223,9 +223,9 @@ __device__ __forceinline__ void jacobi_sweep_warm(V (&A)[NS][NS], V (&U)[NS][NS]
       V t, c, sn;
       if (small) {
 #pragma unroll
-        for (int l = 0; l < L; ++l) {  // (a zero a_pq gives t = 0, also where d = 0)
+        for (int l = 0; l < L; ++l) {  // (|a_pq| <= 2^-12 |d|, so a subnormal d turns nothing)
           const float q = div_normal(ln(apq, l), ln(d, l));
-          ln(t, l) = ln(apq, l) == 0.0f ? 0.0f : q;
+          ln(t, l) = fabsf(ln(d, l)) < 0x1p-126f ? 0.0f : q;
         }
         sn = t;
       } else {
@@ -233,13 +233,14 @@ __device__ __forceinline__ void jacobi_sweep_warm(V (&A)[NS][NS], V (&U)[NS][NS]
         const V r2 = vfma(d, d, vmul(twoa, twoa));
 #pragma unroll
         for (int l = 0; l < L; ++l) {
-          // d + sgn(d) sqrt(d^2 + 4 a_pq^2) is never 0 unless a_pq = 0 (then t = 0;
-          // gap and coupling both below 1e-19, thirteen orders under the degeneracy
-          // threshold, also give t = 0)
+          // d + sgn(d) sqrt(d^2 + 4 a_pq^2) is at least 2^-63, except where that sum
+          // of squares has left the normal range (gap and coupling below 1e-19,
+          // thirteen orders under the degeneracy threshold): then t = 0, where the
+          // quotient would be 0 / 0
           const float rl = ln(r2, l);
           const float den = ln(d, l) + copysignf(rl * rsqrt_normal(rl), ln(d, l));
           const float q = div_normal(ln(twoa, l), den);
-          ln(t, l) = ln(apq, l) == 0.0f ? 0.0f : q;
+          ln(t, l) = rl < 0x1p-126f ? 0.0f : q;
         }
         const V tt1 = vfma(t, t, splat<V>(1.0f));
 #pragma unroll
