@@ -197,8 +197,11 @@ __device__ __forceinline__ double int_double(uint32_t i) {
   return __dadd_rn(__hiloint2double(0x43300000, (int)i), -0x1p52);
 }
 
-// 1 / sqrt(x) for x in the normal range: the hardware approximation y (relative
-// error e/2, e = 1 - x y^2) and one third-order step y (1 + e/2 + 3/8 e^2).
+// 1 / sqrt(x) for x in the normal range: the hardware approximation y and one
+// third-order step.  With e = 1 - x y^2 the root is y (1 - e)^(-1/2), of which the
+// binomial series gives y (1 + e/2 + 3/8 e^2); the first term left out is 5/16 e^3,
+// below 2^-56 of y.  Within 2^-52 of the root (a test: every exponent from -500 to
+// 500).
 __device__ __forceinline__ double rsqrt64(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));

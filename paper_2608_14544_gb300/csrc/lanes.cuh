@@ -55,10 +55,10 @@ template <typename V>
 __device__ __forceinline__ V vsub(V a, V b) { return vfma(b, splat<V>(-1.0f), a); }
 
 // The hardware reciprocal square root, reciprocal and approximate quotient
-// without the library forms' rescaling of subnormal operands (two to five more
-// instructions each): for normal operands and results the same bits as
-// rsqrtf (compared on every positive normal float) and __fdividef (compared on
-// 2^31 random pairs); subnormals count as zero.
+// without the library forms' handling of subnormal operands: for normal operands
+// and results the same bits as rsqrtf (every positive normal float) and as
+// __fdividef (2^30 random pairs), both compared by a test; subnormals count as
+// zero.
 __device__ __forceinline__ float rsqrt_normal(float x) {
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -74,8 +74,8 @@ __device__ __forceinline__ float div_normal(float a, float b) {
   asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
   return r;
 }
-// 1 / d correctly rounded for an integer 1 <= d <= 2^24 (one Newton step on the
-// hardware reciprocal; equal to __frcp_rn at every such d).
+// 1 / d correctly rounded for an integer 1 <= d <= 2^24: one Newton step r + r (1 -
+// d r) on the hardware reciprocal (a test compares it with __frcp_rn at every d).
 __device__ __forceinline__ float rcp_integer(float d) {
   const float r = rcp_approx(d);
   return __fmaf_rn(r, __fmaf_rn(-d, r, 1.0f), r);
