@@ -1,7 +1,7 @@
 """Benchmark: trajectory-steps/s of the FP32-bulk QCL ensemble propagation in
 its served form, on the 3-mode ohmic spin-boson workload (1e7 walkers, 2000
-steps, outputs every 10 steps), beside the plain FP64 one-launch-per-step
-comparator, the FP64 CPU oracle, the other configurations and the served mix.
+steps, outputs every 10 steps), beside the plain FP64 comparator, the FP64 CPU
+oracle, the other configurations and the served mix.
 
 One timed step = one complete solve submitted to the request server
 (qcl_server_submit / qcl_server_wait): model upload, initial Wigner sample,

@@ -192,7 +192,8 @@ qcl_status qcl_sample_initial(const qcl_model* model, const qcl_ensemble_desc* e
  * (32-walker groups, tiles of qcl_shard_tile_walkers walkers, tiles in index
  * order), so that results do not depend on the launch shape and two calls give
  * the same bits as one.  An FP64 launch runs the steps of up to three output
- * times or 256 steps (two states), or up to 16 steps (more states); FP32-bulk
+ * times or 256 steps (two states), or up to 16 steps (more states), fewer where
+ * that would take longer than about a quarter of a second; FP32-bulk
  * ensembles run a persistent kernel over the tiles with state held in
  * registers (two-state models of 33..256 modes split each walker's modes over
  * 2 or 4 warps, so their tiles hold 128 or 64 walkers).  N_s-state models

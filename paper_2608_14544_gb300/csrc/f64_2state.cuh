@@ -1,5 +1,5 @@
-// f64_2state.cuh -- device code of the FP64 two-state walker shared by the
-// one-launch-per-step kernels (kernels_f64.cu) and the spawning kernels
+// f64_2state.cuh -- device code of the FP64 two-state walker shared by the step
+// kernels (kernels_f64.cu: many steps a launch) and the spawning kernels
 // (spawn.cu): SoA views, the closed-form decomposition, the half kicks, one
 // whole step of one walker (Verlet, phase, transition test) and the walker's
 // observable contributions.
@@ -29,11 +29,10 @@ __device__ __forceinline__ W64 view64(void* buf, int64_t nt, int ns, int n) {
 }
 
 // Closed-form two-state decomposition at R: W = s + a sigma_z + b sigma_x,
-// r = |(a, b)|, cos 2theta = a/r, sin 2theta = b/r (theta = atan2(b, a)/2, with
-// theta = 0 at r = 0); the eigenvector angle (c, s) = (cos theta, sin theta) by
-// the cancellation-free half-angle formulas.
+// r = |(a, b)|, theta = atan2(b, a)/2 (0 at r = 0); the eigenvector angle (c, s) =
+// (cos theta, sin theta) by the cancellation-free half-angle formulas.
 struct Ad2 {
-  double a, b, r, c2, s2;
+  double a, b, r;
 };
 
 __device__ __forceinline__ void half_angle(const Ad2& d, double& c, double& s) {

@@ -1,6 +1,6 @@
-// nstate_f64.cuh -- the FP64 path of N_s-state models: sampling, one launch
-// per output time (adiabatic and diabatic), observation and trajectory spawning, in
-// the oracle's operation order (its units are compiled without multiply-add
+// nstate_f64.cuh -- the FP64 path of N_s-state models: sampling, steps (adiabatic
+// and diabatic, at most 16 a launch), observation and trajectory spawning, in the
+// oracle's operation order (its units are compiled without multiply-add
 // contraction).
 #pragma once
 #include "nstate_common.cuh"
