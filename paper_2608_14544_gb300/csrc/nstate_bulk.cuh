@@ -851,9 +851,26 @@ __global__ void __launch_bounds__(128, (BulkNMinBlocks<NS, NPL, WPT>::value))
 // events, quarter turns and 24-bit thresholds).  The observation diagonalises
 // W(R) afresh at output times (Jacobi, the sampler's conventions) for the
 // adiabatic block.
+//
+// The 32-mode form takes its coefficients 8 bytes past a 16-byte boundary: there
+// 300011 walkers of three states and 9 to 32 modes took 0.50 ms for 40 steps, on the
+// boundary 0.57, with the same registers.  (The narrower forms, and the two-state
+// kernels, are 3 to 8 % faster on it.)
+template <bool SHIFTED>
+struct CoefArg {
+  CoefN c;
+};
+template <>
+struct CoefArg<true> {
+  uint32_t shift[2];
+  CoefN c;
+};
 template <int NS, int NPL>
 __global__ void __launch_bounds__(128, (NPL > 8 || NS > 5) ? 2 : 4)
-    k_bulkN_dia(const BulkParams bp, const CoefN cf, void* buf, double* __restrict__ part) {
+    k_bulkN_dia(const BulkParams bp, const CoefArg<(NPL > 8)> ca, void* buf,
+                double* __restrict__ part) {
+  static_assert(sizeof(BulkParams) % 16 == 0 && alignof(CoefN) == 4, "the coefficients' places");
+  const CoefN& cf = ca.c;
   constexpr int NN = NS * NS, NTRI = NS * (NS + 1) / 2;
   constexpr int NP = (4 * NN + 15) / 16;
   constexpr int TW = 128;

@@ -108,9 +108,12 @@ struct NStateOps {
                                  : (size_t)SM * bp.n * 128 * sizeof(float);
     const size_t dyn_max = NM == 0 ? ModeRow<NS>::bytes(kMaxN) : (size_t)64 * 128 * sizeof(float);
     if constexpr (NM == 0) {
-      if (bp.repr == QCL_REPR_DIABATIC)
+      if (bp.repr == QCL_REPR_DIABATIC) {
+        CoefArg<(NPL > 8)> ca{};
+        ca.c = cf;
         return launch_persistent(k_bulkN_dia<NS, NPL>, per_sm[1], n_sm[1], bp, grid_cap, 1, dyn,
-                                 dyn_max, st, bp, cf, buf, part);
+                                 dyn_max, st, bp, ca, buf, part);
+      }
     }
     if constexpr (NPL == 0 && NM == 0 && NS <= 4) {
       return 0;  // (adiabatic models of N_s <= 4 take NM > 0)
