@@ -194,11 +194,24 @@ struct NStateOps {
     // at 128 modes P alone left two, and was 40 % slower than no arrays).
     // N_s = 4, 300011 walkers x 30 steps: 12 modes 0.81 -> 0.74 ms, 32 modes
     // 1.53 -> 1.25, 64 modes 2.72 -> 2.29, 128 modes 5.63 -> 5.13.
+    // Ensembles of one turn (at most four tiles on every SM) wait for one walker's
+    // chain instead, and their R and P stay in L1: the form without arrays is
+    // faster there, for N_s = 4 from 24 modes and N_s = 3 from 48.  N_s = 4, 40
+    // steps, arrays / none: 3000 walkers 32 modes 233 / 200 us, 64 modes 524 / 342;
+    // 77824 walkers 436 / 398 and 703 / 645; 100001 walkers 630 / 695 and 1338 /
+    // 1417.  N_s = 3, 3000 walkers, 40 modes 189 / 195, 48 modes 252 / 223.
     if constexpr (NS <= 4) {
       if (mem && bp.repr != QCL_REPR_DIABATIC) {
+        static const int n_sm = [] {
+          int dev = 0, n = 0;
+          cudaGetDevice(&dev);
+          cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+          return n;
+        }();
+        const bool one_turn = bp.n >= (NS == 4 ? 24 : 48) && bp.n_tiles <= 4 * (int64_t)n_sm;
+        if (bp.n > 64 || one_turn) return bulk_npl<0, 1, 256, 0>(bp, cf, mh, buf, part, grid_cap, st);
         if (bp.n <= 32) return bulk_npl<0, 1, 64, 2>(bp, cf, mh, buf, part, grid_cap, st);
-        if (bp.n <= 64) return bulk_npl<0, 1, 64, 1>(bp, cf, mh, buf, part, grid_cap, st);
-        return bulk_npl<0, 1, 256, 0>(bp, cf, mh, buf, part, grid_cap, st);
+        return bulk_npl<0, 1, 64, 1>(bp, cf, mh, buf, part, grid_cap, st);
       }
     }
     if (mem) return bulk_npl<0>(bp, cf, mh, buf, part, grid_cap, st);
