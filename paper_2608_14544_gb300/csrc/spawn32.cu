@@ -294,13 +294,13 @@ __device__ __forceinline__ void add_counts(unsigned int* cnt, bool fires, int64_
 // the families' starts for the observation (a kernel of its own took 11 us).
 //
 // What bounds it: instruction issue at 1e6 walkers, launch latency below some 1e5
-// (3.8 us a step at 1e3, 5.7 at 1e5).  1e5 initial one-mode walkers growing to 1.57e6 over 400 steps
-// with an output every 10: 7.0 ms of device time; 10.0 ms when every launch
-// evaluated its own step again, 15.9 ms with a step in place, a one-block scan
-// and a scatter.  One cooperative launch for many steps, with a decoupled
-// look-back over the groups' counts and a grid barrier, was slower (13.6 ms): a
-// poll of another die's word costs about a microsecond, and a step needs several
-// in a row.
+// (3.8 us a step at 1e3, 5.7 at 1e5).  1e5 initial one-mode walkers growing to
+// 1.57e6 over 400 steps with an output every 10: 7.0 ms of device time; 10.0 ms
+// when every launch evaluated its own step again, 15.9 ms with a step in place, a
+// one-block scan and a scatter.  One cooperative launch for many steps, with a
+// decoupled look-back over the groups' counts and a grid barrier, was slower (13.6
+// ms): a poll of another die's word costs about a microsecond, and a step needs
+// several in a row.
 template <int NPL, int KIND, bool DIA, bool FIRST>
 __global__ void __launch_bounds__(256, NPL <= 4 ? 3 : (NPL <= 8 ? 2 : 1))
     k_spawn_chain32(const BulkParams bp, const CoefLocal<NPL> cf, const SpawnLayout L, void* buf,
@@ -675,12 +675,13 @@ __device__ __forceinline__ void add_product(f2& a, float x, float f) {
 // neighbouring walkers.  An output of 200000 families by 8, 4, 2 and 1: 13.8
 // walkers of 32 modes 411, 338, 348 and 378 us, 5.2 of 40 modes 273, 230, 203 and
 // 215, 5.4 of 100 modes 689, 567, 492 and 458; of 16 modes 203, 206, 223 and 244.
-// 32 / w families go side by side, the
-// block's families ordered by size so that those of a warp are alike and few
-// lanes idle, and the block's warps take such groups in turn, widest first.  The
-// X of the tile's families then meet in shared memory, where the even lane of a
-// pair adds X, the odd lane X^2, of one quantity over a warp's 32 families in
-// order, and the 8 warps are folded by the fixed tree of the observation kernels.
+//
+// 32 / w families go side by side, the block's families ordered by size so that
+// those of a warp are alike and few lanes idle, and the block's warps take such
+// groups in turn, widest first.  The X of the tile's families then meet in shared
+// memory, where the even lane of a pair adds X, the odd lane X^2, of one quantity
+// over a warp's 32 families in order, and the 8 warps are folded by the fixed tree
+// of the observation kernels.
 //
 // A family of more than kFamWide walkers is taken by the whole block (a walker of
 // 256 a lane, the warps' pairs added in order), so that the few large families of
