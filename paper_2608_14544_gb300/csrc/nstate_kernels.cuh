@@ -57,24 +57,28 @@ struct NStateOps {
     k_spawnN_sample32<NS><<<(unsigned)(nb > 0 ? nb : 1), 128, 0, st>>>(sp, cap, buf);
     launches_add(1);
   }
+  // (false: the launch was refused)
   template <int NPL>
-  static void spawn_step32_npl(const BulkParams& bp, const CoefN& cf, void* buf, int64_t cap,
+  static bool spawn_step32_npl(const BulkParams& bp, const CoefN& cf, void* buf, int64_t cap,
                                int64_t n0, int64_t step, cudaStream_t st) {
     // (NPL = 0: the mode table in dynamic shared memory)
     size_t dyn = 0;
     if constexpr (NPL == 0) {
       dyn = ModeRow<NS>::bytes(bp.n);
-      if (!allow_dynamic_shared(k_spawnN_step32<NS, NPL>, ModeRow<NS>::bytes(kMaxN))) return;
+      if (!allow_dynamic_shared(k_spawnN_step32<NS, NPL>, ModeRow<NS>::bytes(kMaxN))) return false;
     }
     k_spawnN_step32<NS, NPL><<<spawn_grid(cap), 256, dyn, st>>>(bp, cf, buf, cap, n0, step);
+    return true;
   }
   // one FP32 spawning step (step kernel, scan, scatter): up to 8 modes in
   // registers, beyond (or under the modes-in-memory option) in memory
   static int spawn_step32(const BulkParams& bp, const CoefN& cf, void* buf, int64_t cap,
                           int64_t n0, int64_t step0, int64_t step, cudaStream_t st) {
-    if (cf.modes_in_memory == 1 || bp.n > 8) spawn_step32_npl<0>(bp, cf, buf, cap, n0, step, st);
-    else if (bp.n <= 4) spawn_step32_npl<4>(bp, cf, buf, cap, n0, step, st);
-    else spawn_step32_npl<8>(bp, cf, buf, cap, n0, step, st);
+    // (without the step's counts nothing may be scanned or scattered)
+    if (!(cf.modes_in_memory == 1 || bp.n > 8 ? spawn_step32_npl<0>(bp, cf, buf, cap, n0, step, st)
+          : bp.n <= 4 ? spawn_step32_npl<4>(bp, cf, buf, cap, n0, step, st)
+                      : spawn_step32_npl<8>(bp, cf, buf, cap, n0, step, st)))
+      return 0;
     launch_spawn_scan(buf, cap, bp.n, n0, QCL_PREC_FP32_BULK, NS, step0, step, st);
     k_spawnN_scatter32<NS><<<spawn_grid(cap), 256, 0, st>>>(buf, cap, bp.n, n0, step0, step,
                                                             bp.seed);

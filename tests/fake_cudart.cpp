@@ -31,6 +31,7 @@ std::vector<Launch> launches;
 thread_local int device = 0;
 thread_local std::vector<Config> configs;
 thread_local cudaError_t last = cudaSuccess;
+bool refuse = false;  // cudaFuncSetAttribute fails
 
 cudaError_t set(cudaError_t e) {
   if (e != cudaSuccess) last = e;
@@ -58,6 +59,7 @@ void fake_reset() {
   std::lock_guard<std::mutex> lock(mu);
   launches.clear();
 }
+void fake_refuse_limits(int on) { refuse = on != 0; }
 long fake_count(const char* part) {
   std::lock_guard<std::mutex> lock(mu);
   long n = 0;
@@ -108,7 +110,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
   return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes);
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
-  if (a != cudaFuncAttributeMaxDynamicSharedMemorySize || v < 0 || v > (227 << 10))
+  if (refuse || a != cudaFuncAttributeMaxDynamicSharedMemorySize || v < 0 || v > (227 << 10))
     return set(cudaErrorInvalidValue);
   std::lock_guard<std::mutex> lock(mu);
   limits[{f, device}] = v;

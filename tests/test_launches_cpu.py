@@ -95,6 +95,26 @@ def test_spawning_on_a_second_device(fake, ns, n):
         lib.cudaSetDevice(0)
 
 
+def test_a_refused_limit_is_the_calls_error(fake):
+    """No kernel runs in place of the refused one, and none on what it would have
+    written."""
+    q, lib = fake
+    lib.fake_refuse_limits(1)
+    try:
+        lib.fake_reset()
+        spawn = q.SpawnRun(q.Model(_lvc(8, 256)), 100, 1000, 1, 3, precision=q.PREC_FP32_BULK)
+        with pytest.raises(q.QclError, match="launch failed"):
+            spawn.propagate(1, 0.01, 2)
+        assert lib.fake_count(b"k_spawn_scan") == lib.fake_count(b"k_spawnN_scatter32") == 0
+        for model in (_lvc(4, 64), wl.spin_boson(0.5, 0.5, *wl.ohmic_modes(100, 0.3, 2.5))):
+            run = q.Run(q.Model(model), 300_000, 1, q.PREC_FP32_BULK, 3)
+            with pytest.raises(q.QclError, match="launch failed"):
+                run.propagate(4, 0.01, 2)
+        assert lib.fake_count(b"k_bulk") == 0
+    finally:
+        lib.fake_refuse_limits(0)
+
+
 @pytest.mark.parametrize("ns,n,rep,walkers,steps,least,most", [
     (2, 1, "adiabatic", 10_000, 600, 3, 3), (2, 3, "adiabatic", 1_000_000, 512, 2, 2),
     (2, 256, "adiabatic", 10_000_000, 256, 100, 256), (2, 100, "diabatic", 3_000_000, 256, 5, 64),
